@@ -1,6 +1,7 @@
 // dpde_api.cu -- the C ABI of include/dpde.h: handle, buffers, launch
 // sequence of one timestep, CUDA-graph replay, observables, diagnostics.
 #include "dpde.h"
+#include "dpde_force.cuh"
 #include "dpde_ssa_levels.cuh"
 #include "dpde_ssa_persistent.cuh"
 
@@ -71,8 +72,8 @@ struct dpde_handle {
     // projection on the internal energies (Sec. IV.C)
     bool project = false;
     double *proj_e0 = nullptr, *proj_shift = nullptr, *proj_partial = nullptr;
-    void *eA = nullptr, *eB = nullptr, *nbr_w = nullptr, *fwd_w = nullptr, *fwd_g = nullptr;
-    int *cA = nullptr, *cB = nullptr, *nbr_j = nullptr, *nbr_n = nullptr, *fwd_j = nullptr, *fwd_n = nullptr;
+    void *eA = nullptr, *eB = nullptr, *nbr = nullptr, *fwd_g = nullptr;
+    int *cA = nullptr, *cB = nullptr, *nbr_n = nullptr, *fwd_n = nullptr;
     int4 *tile_org = nullptr, *tile_dim = nullptr;
     int ntiles = 0;
     // SSA colour classes: cells grouped by colour index (col_z * 5 + col_y) * 5
@@ -110,13 +111,13 @@ struct dpde_handle {
     long long wait_budget = 2000000000ll;
     int ssa_group = 0;        // bricks per warp; 0 = dom_group_auto
     int dom_group_auto = 1;   // 32 / the largest class of a brick, in 1..SSA_GROUP_MAX
-    int hcap = 0;             // halo particles staged per force tile
-    int hcap_dense = 0;       // ... per deferred (dense) tile
-    size_t tile_smem_dense = 0;
+    ForceShape tile_shape{}, tile_shape_dense{};   // shared-memory shapes of the two force launches
+    int tile_warps = 0, tile_warps_dense = 0;   // warps per block of the two force launches
+    FrameTiles frames{};      // frame tiles of the force pass
+    int4* frame_org = nullptr;
+    unsigned char* frame_rel = nullptr;
     int* defer = nullptr;     // deferred tiles of the force pass: list, then count
     int ndense_blocks = 0;
-    int hcc = 0;              // halo cells per force tile, (tile_edge + 2)^3
-    size_t tile_smem = 0;
     double per_cell_max = 0;  // mean particles per cell of the densest replica
     // tuning (dpde_set_tuning / dpde_autotune)
     int tile_edge = TILE_EDGE;
@@ -171,8 +172,8 @@ Ctx<T> make_ctx(dpde_handle* h) {
     C.upot = (T*)h->upot;
     C.key = h->key; C.tmp = h->tmp;
     C.count = h->cnt; C.fill = h->cnt + h->ncells; C.start = h->start;
-    C.nbr_j = h->nbr_j; C.nbr_w = (T*)h->nbr_w; C.nbr_n = h->nbr_n; C.nbr_cap = h->nbr_cap;
-    C.fwd_j = h->fwd_j; C.fwd_w = (T*)h->fwd_w; C.fwd_g = (vec_t<T>*)h->fwd_g; C.fwd_n = h->fwd_n;
+    C.nbr = (ListEnt<T>*)h->nbr; C.nbr_n = h->nbr_n; C.nbr_cap = h->nbr_cap;
+    C.fwd = C.nbr + (size_t)h->nbr_cap * std::max(1, h->N); C.fwd_g = (vec_t<T>*)h->fwd_g; C.fwd_n = h->fwd_n;
     C.rep_of_slot = h->rep_of_slot; C.rep_of_cell = h->rep_of_cell;
     C.brick_rep = h->brick_rep; C.tab = h->tab;
     C.reps = h->d_reps; C.step = h->d_step; C.status = h->d_status; C.wall = h->wallpos;
@@ -216,21 +217,23 @@ void enqueue_sort(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T half_dt, T
     k_scan_add<<<ceil_div(h->ncells, 256), 256, 0, st>>>(h->start, h->bsum, h->ncells, h->N);
     phase(h, st, DPDE_PHASE_SCAN, 1);
     phase(h, st, DPDE_PHASE_GATHER, 0);
-    k_scatter<T><<<nb, h->block, 0, st>>>(C);
+    k_scatter<T><<<nb + ceil_div(h->frames.n, h->block / 32), h->block, 0, st>>>(C, h->frames, nb);
     k_rank_gather<T><<<nb, h->block, 0, st>>>(C);
     phase(h, st, DPDE_PHASE_GATHER, 1);
 }
 
 template <class T>
 void enqueue_force(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T half_dt, int kick, int list) {
-    const dim3 g(h->ntiles), blk(TILE_THREADS), gd(h->ndense_blocks);
+    const dim3 g(h->ntiles), blk(32 * h->tile_warps), gd(h->ndense_blocks), bd(32 * h->tile_warps_dense);
+    const size_t sm = force_smem<T>(h->tile_shape, h->tile_warps),
+                 smd = force_smem<T>(h->tile_shape_dense, h->tile_warps_dense);
     int* cnt = h->defer + h->ntiles;
     cudaMemsetAsync(cnt, 0, sizeof(int), st);
-#define DPDE_FORCE(LMV)                                                                                          \
-    k_force_tile<T, LMV><<<g, blk, h->tile_smem, st>>>(C, h->tile_org, h->tile_dim, half_dt, kick, h->hcap,      \
-                                                       h->hcc, h->defer, cnt);                                   \
-    k_force_tile_dense<T, LMV><<<gd, blk, h->tile_smem_dense, st>>>(C, h->tile_org, h->tile_dim, half_dt, kick, \
-                                                                    h->hcap_dense, h->hcc, h->defer, cnt)
+#define DPDE_FORCE(LMV)                                                                                           \
+    k_force_tile<T, LMV><<<g, blk, sm, st>>>(C, h->tile_org, h->tile_dim, half_dt, kick, h->tile_shape,           \
+                                             h->frames, h->defer, cnt);                                           \
+    k_force_tile_dense<T, LMV><<<gd, bd, smd, st>>> (C, h->tile_org, h->tile_dim, half_dt, kick,                  \
+                                                     h->tile_shape_dense, h->frames, h->defer, cnt)
     switch (list) {
     case LIST_ALL: DPDE_FORCE(LIST_ALL); break;
     case LIST_CROSS: DPDE_FORCE(LIST_CROSS); break;
@@ -525,8 +528,8 @@ void free_all(dpde_handle* h) {
             if (ev) cudaEventDestroy(ev);
     for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
     h->graphs.clear();
-    void* bufs[] = {h->qA, h->pA, h->qB, h->pB, h->F, h->dp, h->upot, h->proj_e0, h->proj_shift, h->proj_partial, h->eA, h->eB, h->nbr_w, h->cA, h->cB, h->nbr_j,
-                    h->nbr_n, h->fwd_j, h->fwd_w, h->fwd_g, h->fwd_n, h->tile_org, h->tile_dim, h->defer, h->col_cells[0], h->col_cells[1], h->dom_cells, h->dom_off, h->dom_cell0, h->rdom_cells, h->rdom_off, h->rdom_cell0, h->lv_off, h->lv_n, h->ssa_defer, h->d_col_off[0], h->d_col_off[1], h->d_bar, h->wallpos, h->idB, h->key, h->tmp, h->cnt, h->start, h->bsum, h->rep_of_slot,
+    void* bufs[] = {h->qA, h->pA, h->qB, h->pB, h->F, h->dp, h->upot, h->proj_e0, h->proj_shift, h->proj_partial, h->eA, h->eB, h->nbr, h->cA, h->cB,
+                    h->nbr_n, h->fwd_g, h->fwd_n, h->tile_org, h->tile_dim, h->frame_org, h->frame_rel, h->defer, h->col_cells[0], h->col_cells[1], h->dom_cells, h->dom_off, h->dom_cell0, h->rdom_cells, h->rdom_off, h->rdom_cell0, h->lv_off, h->lv_n, h->ssa_defer, h->d_col_off[0], h->d_col_off[1], h->d_bar, h->wallpos, h->idB, h->key, h->tmp, h->cnt, h->start, h->bsum, h->rep_of_slot,
                     h->rep_of_cell, h->brick_rep, h->tab, h->chunk_rep, h->chunk_begin, h->chunk_end,
                     h->rep_chunk_begin, h->partial, h->obs_out, h->d_reps, h->d_step, h->d_status,
                     h->staging, h->cells_out};
@@ -542,43 +545,113 @@ void free_all(dpde_handle* h) {
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 
-// Force tiles of edge `edge` cells over every replica, their halo staging
-// capacity (1.08x the mean halo count of the densest replica + 64, over 3
-// standard deviations of a uniform fluid's count) and shared memory size.
+// Force tiles: frame tiles of `edge` cells over every replica, each cut into
+// work tiles of wx x wy x wz cells (the tiles of the launch).
 int set_tiles(dpde_handle* h, int edge) {
-    std::vector<int4> torg, tdim;
+    int dev = 0, nsm = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    // hframe: 2.5x the mean halo of the densest replica's frame tiles, as far
+    // as 224 KB of shared memory would hold it (28 or 44 bytes a particle,
+    // 12 a cell); beyond, separations are formed cell by cell
+    const size_t tper = h->mixed ? 28 : 44;
+    const int hcc = (edge + 2) * (edge + 2) * (edge + 2);
+    const size_t thead = ((size_t)(3 * hcc + 67) * 4 + 28 * 256 * 2 + 31) & ~(size_t)31;
+    const double mean_frame = h->per_cell_max * hcc;
+    const int fit = (int)std::min<double>(std::min<double>(1.08 * mean_frame + 64.0, 65535.0),
+                                          (double)((200 * 1024 - thead) / tper)) & ~3;
+    const int hframe = std::max(fit, (int)std::min<double>(std::min<double>(2.5 * mean_frame + 64.0, 65535.0),
+                                                    (double)((224 * 1024 - thead) / tper))) & ~3;
+    // work tile: edge x edge x 2 cells in a single box (the least halo per
+    // own particle: force pass 720 us at 4M against 800 us with 3 x 3 x 3),
+    // 3 x 3 x 3 in a batch, whose smaller boxes the frames cut into narrow
+    // remainders (256 boxes of 2,000 to 64,000: 1085 us against 1240 us). Its
+    // longest edge is halved while the mean halo takes more than ~1/4 of an
+    // SM's shared memory or the launch has fewer than six blocks per SM
+    // (108,000 particles: 43 -> 38 us with the first halving).
+    int w[3] = {edge, edge, std::min(2, edge)};
+    if (h->R > 1) w[0] = w[1] = w[2] = (edge + 1) / 2;
+    auto count = [&]() {
+        long long n = 0;
+        for (const RepInfo& I : h->info) {
+            long long m = 1;
+            for (int a = 0; a < 3; ++a) {
+                long long k = 0;
+                for (int f = 0; f < I.nc[a]; f += edge) k += ceil_div(std::min(edge, I.nc[a] - f), w[a]);
+                m *= k;
+            }
+            n += m;
+        }
+        return n;
+    };
+    auto shape = [&](double halo) {
+        ForceShape S;
+        S.hcap = (int)std::min(halo, 65000.0) & ~3;
+        S.nhc = (w[0] + 2) * (w[1] + 2) * (w[2] + 2);
+        S.noc = w[0] * w[1] * w[2];
+        S.wide = mean_frame > 0.5 * hframe;   // some frame tile may go cell by cell
+        return S;
+    };
+    auto warps = [&](double over) {   // for the mean own particles, times `over`
+        const double own = h->per_cell_max * w[0] * w[1] * w[2] * over;
+        return std::max(2, std::min(FORCE_WARPS_MAX, (int)std::ceil(own / 32.0)));
+    };
+    auto bytes = [&](const ForceShape& S, double over = 1.08) {
+        return h->mixed ? force_smem<float>(S, warps(over)) : force_smem<double>(S, warps(over));
+    };
+    auto mean_halo = [&]() { return h->per_cell_max * (w[0] + 2) * (w[1] + 2) * (w[2] + 2); };
+    const size_t budget = h->mixed ? 56 * 1024 : 74 * 1024;
+    for (;;) {
+        const bool big = bytes(shape(1.08 * mean_halo() + 64.0)) > budget;
+        const bool few = count() < 6 * nsm && h->per_cell_max * w[0] * w[1] * w[2] > 24.0;
+        const int a = w[1] >= w[0] && w[1] >= w[2] ? 1 : (w[0] >= w[2] ? 0 : 2);
+        if (!(big || few) || w[a] == 1) break;
+        w[a] = (w[a] + 1) / 2;
+    }
+    const size_t smem_limit = 200 * 1024;
+    // regular capacity 1.08x the mean halo + 64 (over 4 standard deviations
+    // of a uniform fluid's count), deferred tiles 2.5x the mean
+    auto capped = [&](double halo) {
+        ForceShape S = shape(halo);
+        while (S.hcap > 64 && bytes(S, 1.7) > smem_limit) S.hcap = (S.hcap * 15 / 16) & ~3;
+        return S;
+    };
+    const ForceShape S0 = capped(1.08 * mean_halo() + 64.0), S1 = capped(2.5 * mean_halo() + 128.0);
+    const size_t smem = bytes(S0), smem_dense = bytes(S1, 1.7);
+    std::vector<int4> torg, tdim, forg;
     for (int r = 0; r < h->R; ++r) {
         const RepInfo& I = h->info[r];
-        for (int z0 = 0; z0 < I.nc[2]; z0 += edge)
-            for (int y0 = 0; y0 < I.nc[1]; y0 += edge)
-                for (int x0 = 0; x0 < I.nc[0]; x0 += edge) {
-                    torg.push_back(make_int4(r, x0, y0, z0));
-                    tdim.push_back(make_int4(std::min(edge, I.nc[0] - x0), std::min(edge, I.nc[1] - y0),
-                                             std::min(edge, I.nc[2] - z0), 0));
+        const int f0 = (int)forg.size(), fnx = ceil_div(I.nc[0], edge), fny = ceil_div(I.nc[1], edge);
+        for (int z = 0; z < I.nc[2]; z += edge)
+            for (int y = 0; y < I.nc[1]; y += edge)
+                for (int x = 0; x < I.nc[0]; x += edge) forg.push_back(make_int4(r, x, y, z));
+        std::vector<std::pair<int, int>> cut[3];   // work-tile starts and sizes along each axis
+        for (int a = 0; a < 3; ++a)
+            for (int f = 0; f < I.nc[a]; f += edge)
+                for (int o = f; o < std::min(f + edge, I.nc[a]); o += w[a])
+                    cut[a].push_back({o, std::min(w[a], std::min(f + edge, I.nc[a]) - o)});
+        for (const auto& z : cut[2])
+            for (const auto& y : cut[1])
+                for (const auto& x : cut[0]) {
+                    torg.push_back(make_int4(r, x.first, y.first, z.first));
+                    tdim.push_back(make_int4(x.second, y.second, z.second,
+                                             f0 + (z.first / edge * fny + y.first / edge) * fnx + x.first / edge));
                 }
     }
-    const int hcc = (edge + 2) * (edge + 2) * (edge + 2);
-    const size_t thead = tile_head_bytes(hcc);
-    const size_t tper = h->mixed ? tile_per_particle<float>() : tile_per_particle<double>();
-    const double mean_halo = h->per_cell_max * hcc;
-    const size_t smem_limit = 200 * 1024;
-    int hcap = (int)std::min<double>(std::min<double>(1.08 * mean_halo + 64.0, 65535.0),
-                                     (double)((smem_limit - thead) / tper));
-    hcap &= ~3;   // keeps the arrays after the positions 16-byte aligned
-    const size_t smem = 32 + thead + (size_t)hcap * tper;
-    // deferred tiles: 2.5x the mean halo (dense regions such as a shock front)
-    int hcap_dense = (int)std::min<double>(std::min<double>(2.5 * mean_halo + 64.0, 65535.0),
-                                           (double)((smem_limit + 24 * 1024 - thead) / tper));
-    hcap_dense = std::max(hcap_dense, hcap) & ~3;
-    const size_t smem_dense = 32 + thead + (size_t)hcap_dense * tper;
     if (h->tile_org) cudaFree(h->tile_org);
     if (h->tile_dim) cudaFree(h->tile_dim);
     if (h->defer) cudaFree(h->defer);
-    h->tile_org = h->tile_dim = nullptr;
+    if (h->frame_org) cudaFree(h->frame_org);
+    if (h->frame_rel) cudaFree(h->frame_rel);
+    h->tile_org = h->tile_dim = h->frame_org = nullptr;
+    h->frame_rel = nullptr;
     h->defer = nullptr;
     CK(h, cudaMalloc(&h->defer, sizeof(int) * (torg.size() + 1)));
     CK(h, cudaMalloc(&h->tile_org, sizeof(int4) * std::max<size_t>(1, torg.size())));
     CK(h, cudaMalloc(&h->tile_dim, sizeof(int4) * std::max<size_t>(1, tdim.size())));
+    CK(h, cudaMalloc(&h->frame_org, sizeof(int4) * std::max<size_t>(1, forg.size())));
+    CK(h, cudaMalloc(&h->frame_rel, std::max<size_t>(1, forg.size())));
+    CK(h, cudaMemcpy(h->frame_org, forg.data(), sizeof(int4) * forg.size(), cudaMemcpyHostToDevice));
+    CK(h, cudaMemset(h->frame_rel, 0, std::max<size_t>(1, forg.size())));
     CK(h, cudaMemcpy(h->tile_org, torg.data(), sizeof(int4) * torg.size(), cudaMemcpyHostToDevice));
     CK(h, cudaMemcpy(h->tile_dim, tdim.data(), sizeof(int4) * tdim.size(), cudaMemcpyHostToDevice));
     const int sm = (int)smem, smd = (int)smem_dense;
@@ -603,18 +676,13 @@ int set_tiles(dpde_handle* h, int edge) {
         CK(h, cudaFuncSetAttribute(k_force_tile_dense<double, LIST_FWD>, A, smd));
     }
     h->ntiles = (int)torg.size();
-    h->hcc = hcc;
-    h->hcap = hcap;
-    h->tile_smem = smem;
-    h->hcap_dense = hcap_dense;
-    h->tile_smem_dense = smem_dense;
-    int nsm = 152;
-    {
-        int dev = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess)
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    }
-    h->ndense_blocks = std::max(1, std::min((int)torg.size(), nsm));
+    h->frames = FrameTiles{h->frame_org, h->frame_rel, (int)forg.size(), edge, hframe};
+    h->tile_shape = S0;
+    h->tile_shape_dense = S1;
+    h->tile_warps = warps(1.08);
+    h->tile_warps_dense = warps(1.7);
+    const int per_sm = std::max(1, std::min(4, (int)(227 * 1024 / (smem_dense + 1024))));
+    h->ndense_blocks = std::max(1, std::min((int)torg.size(), nsm * per_sm));
     h->tile_edge = edge;
     return DPDE_OK;
 }
@@ -911,11 +979,8 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
     CKC(cudaMalloc(&h->cA, sizeof(int) * n1));
     CKC(cudaMalloc(&h->cB, sizeof(int) * n1));
     CKC(cudaMalloc(&h->idB, sizeof(uint32_t) * n1));
-    CKC(cudaMalloc(&h->nbr_j, sizeof(int) * n1 * (size_t)h->nbr_cap));
-    CKC(cudaMalloc(&h->nbr_w, tsz * n1 * (size_t)h->nbr_cap));
+    CKC(cudaMalloc(&h->nbr, 2 * 2 * tsz * n1 * (size_t)h->nbr_cap));   // neighbour, then forward lists
     CKC(cudaMalloc(&h->nbr_n, sizeof(int) * n1));
-    CKC(cudaMalloc(&h->fwd_j, sizeof(int) * n1 * (size_t)h->nbr_cap));
-    CKC(cudaMalloc(&h->fwd_w, tsz * n1 * (size_t)h->nbr_cap));
     CKC(cudaMalloc(&h->fwd_g, vsz * n1 * (size_t)h->nbr_cap));
     CKC(cudaMalloc(&h->fwd_n, sizeof(int) * n1));
     CKC(cudaMalloc(&h->key, sizeof(int) * n1));

@@ -228,6 +228,13 @@ template <class T> struct PotT {
 // For 0 < r2 < r_c^2 and ir = 1/sqrt(r2): v(r), fr = -v'(r)/r (so that the
 // force on i is fr (q_i - q_j)) and lap = v''(r) + 2 v'(r)/r.
 template <class T>
+__device__ __forceinline__ void pair_pot_soft(const PotT<T>& P, T r2, T ir, T& v, T& fr, T& lap) {
+    const T w = T(1) - r2 * ir * P.inv_rc;
+    v = P.half_arc * w * w;
+    fr = P.a * w * ir;
+    lap = P.a * P.inv_rc - T(2) * P.a * w * ir;
+}
+template <class T>
 __device__ __forceinline__ void pair_pot(const PotT<T>& P, T r2, T ir, T& v, T& fr, T& lap) {
     const T r = r2 * ir;
     if (P.kind == 1) {
@@ -238,10 +245,7 @@ __device__ __forceinline__ void pair_pot(const PotT<T>& P, T r2, T ir, T& v, T& 
         fr = -dv * ir;
         lap = P.lj4e * (T(156) * s12 - T(42) * s6) * ir2 + T(2) * dv * ir;
     } else {
-        const T w = T(1) - r * P.inv_rc;
-        v = P.half_arc * w * w;
-        fr = P.a * w * ir;
-        lap = P.a * P.inv_rc - T(2) * P.a * w * ir;
+        pair_pot_soft(P, r2, ir, v, fr, lap);
     }
 }
 

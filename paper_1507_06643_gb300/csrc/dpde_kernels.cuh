@@ -13,6 +13,13 @@ namespace dpde {
 
 enum ListMode : int { LIST_NONE = 0, LIST_ALL = 1, LIST_CROSS = 2, LIST_FWD = 3 };
 
+// One entry of a neighbour or forward list: the partner's slot and w = 1 -
+// r / r_cut, written and read as one 8- or 16-byte word.
+template <class T> struct __align__(2 * sizeof(T)) ListEnt {
+    int j;
+    T w;
+};
+
 template <class T> struct Ctx {
     using vec = vec_t<T>;
     using E = eps_t<T>;
@@ -26,13 +33,11 @@ template <class T> struct Ctx {
     int* count;      // per-cell counts (ncells), followed by fill (ncells)
     int* fill;
     int* start;      // ncells + 1 exclusive prefix of count
-    int* nbr_j;      // neighbour list, [k * N + i]
-    T* nbr_w;        // 1 - r/r_cut of each entry
+    ListEnt<T>* nbr; // neighbour list, [k * N + i], nbr_cap rows (fwd follows in the same buffer)
     int* nbr_n;      // entries per particle
     int nbr_cap;
-    int* fwd_j;      // forward pairs of the SSA as the force pass writes them, entry-major
-                     //   [k * N + i], partner slots in SSA sequence order (segment, id)
-    T* fwd_w;        //   w = 1 - r/r_cut of each entry
+    ListEnt<T>* fwd; // forward pairs of the SSA as the force pass writes them, entry-major
+                     //   [k * N + i], in SSA sequence order (segment, id)
     vec* fwd_g;      // (G_it, w) of each entry, particle-major [i * nbr_cap + k] (the SSA
                      //   chains' reading order), drawn before the SSA launches; the level
                      //   records of the SSA by levels; then the SER sweeps' delta p_ij
@@ -79,6 +84,12 @@ __device__ __forceinline__ void check_state(unsigned int* st, const vec_t<T>& p,
     if (!eps_ok(e)) flag(st, ST_NEG_EPS);
     if (!finite3(p) || !eps_finite(e)) flag(st, ST_NONFINITE);
 }
+
+constexpr int NBR_J_BITS = 27;   // particle count limit 2^27 of a handle
+
+template <class T> __device__ __forceinline__ T trsqrt(T x);
+template <> __device__ __forceinline__ float trsqrt(float x) { return rsqrtf(x); }
+template <> __device__ __forceinline__ double trsqrt(double x) { return rsqrt(x); }
 
 // offset * l for a cell offset d in {-1, 0, 1}
 template <class T> __device__ __forceinline__ T shift(int d, T l) {
@@ -410,8 +421,46 @@ __global__ void k_scan_add(int* __restrict__ out, const int* __restrict__ bsum, 
 // counting sort by (cell, id): scatter into cells, then rank by id inside
 // each cell and gather A -> B (refreshing beta = C_v / eps)
 // ---------------------------------------------------------------------------
+// h / n for 0 <= h < 4096, n <= 16, from in = 1 / n: (h + 1/2) / n stays
+// 1/32 clear of the next integer
+__device__ __forceinline__ int small_div(int h, float in) { return (int)(((float)h + 0.5f) * in); }
+
+// Frame tiles: (replica, first cells) of each, and whether its halo holds more
+// particles than the frame is used for (set by k_scatter's last blocks).
+struct FrameTiles {
+    const int4* org;
+    unsigned char* rel;
+    int n, edge, hframe;
+};
+
+// Blocks of the launch beyond the particles' nb count the halos of the force
+// pass's frame tiles, a warp per tile.
 template <class T>
-__global__ void k_scatter(Ctx<T> C) {
+__global__ void k_scatter(Ctx<T> C, FrameTiles F, int nb) {
+    if ((int)blockIdx.x >= nb) {
+        const int f = ((int)blockIdx.x - nb) * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+        if (f >= F.n) return;
+        const int4 o = F.org[f];
+        const RepInfo& R = C.reps[o.x];
+        const int nx = R.nc[0], ny = R.nc[1], nz = R.nc[2];
+        const int HX = min(F.edge, nx - o.y) + 2, HY = min(F.edge, ny - o.z) + 2, HZ = min(F.edge, nz - o.w) + 2;
+        const float iHX = 1.0f / (float)HX, iHY = 1.0f / (float)HY;
+        int sum = 0;
+#pragma unroll 4
+        for (int h = lane; h < HX * HY * HZ; h += 32) {
+            const int row = small_div(h, iHX), hz = small_div(row, iHY);
+            int x = o.y + h - row * HX - 1, y = o.z + row - hz * HY - 1, z = o.w + hz - 1;
+            const bool use = !(R.walls && (z < 0 || z >= nz));   // nothing beyond a wall
+            x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+            y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+            z = z < 0 ? z + nz : (z >= nz ? z - nz : z);
+            const int c = use ? cell_index(C.tab, R, x, y, z) : 0;
+            sum += use ? C.start[c + 1] - C.start[c] : 0;
+        }
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0) F.rel[f] = sum > F.hframe;
+        return;
+    }
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= C.N) return;
     const int c = C.key[s];
@@ -456,404 +505,6 @@ __global__ void k_copy_back(Ctx<T> C) {
     C.eA[s] = ev;
     C.cA[s] = C.cB[s];
     check_state<T>(C.status, pv, ev);
-}
-
-// ---------------------------------------------------------------------------
-// conservative forces F(q) on B (soft repulsion a (1 - r/r_cut) r_hat), the
-// second Verlet half-kick p += dt/2 F when kick != 0, and the lists of the
-// fluctuation/dissipation part:
-//   LIST_ALL   every neighbour (j, w = 1 - r/r_cut)           -> nbr
-//   LIST_CROSS neighbours in another brick                      -> nbr
-//              and forward neighbours in the same brick         -> fwd
-//   LIST_FWD   forward neighbours (whole-replica SSA)           -> fwd
-// A forward neighbour of i lies in the half stencil (segment > 13) or in
-// i's own cell after i. Both force paths visit the neighbour cells in
-// increasing segment s = 9 (dz+1) + 3 (dy+1) + (dx+1) and each cell in slot
-// (= id) order, so a forward row lists i's pairs in SSA sequence order.
-// ---------------------------------------------------------------------------
-constexpr int NBR_J_BITS = 27;   // particle count limit 2^27 of a handle
-
-template <class T> __device__ __forceinline__ T trsqrt(T x);
-template <> __device__ __forceinline__ float trsqrt(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double trsqrt(double x) { return rsqrt(x); }
-
-template <class T>
-struct PairOut {
-    T fx = 0, fy = 0, fz = 0;
-    T u = 0;    // sum of v(r) over the neighbours
-    int nn = 0, nf = 0;
-};
-
-// one neighbour j (global slot) of i at separation d with |d|^2 = r2; fwd
-// tells whether j is a forward neighbour of i, cross whether j's brick
-// differs from i's
-template <class T, int LM>
-__device__ __forceinline__ void force_hit(const Ctx<T>& C, int i, int j, bool fwd, bool cross, T dx, T dy, T dz,
-                                          T r2, PairOut<T>& o) {
-    const size_t N = (size_t)C.N;
-    T w = T(1);
-    if (r2 > T(0)) {
-        const T ir = trsqrt(r2);
-        w = T(1) - r2 * ir * C.inv_rc;
-        T v, fr, lap;
-        pair_pot(C.pot, r2, ir, v, fr, lap);
-        o.fx += fr * dx; o.fy += fr * dy; o.fz += fr * dz;
-        o.u += v;
-    } else {
-        o.u += pair_pot_at_zero(C.pot);
-    }
-    if (LM == LIST_ALL || (LM == LIST_CROSS && cross)) {
-        if (o.nn < C.nbr_cap) {
-            C.nbr_j[(size_t)o.nn * N + i] = j;
-            C.nbr_w[(size_t)o.nn * N + i] = w;
-        }
-        ++o.nn;
-    } else if ((LM == LIST_CROSS || LM == LIST_FWD) && fwd) {
-        if (o.nf < C.nbr_cap) {
-            const size_t at = (size_t)o.nf * N + i;
-            C.fwd_j[at] = j;
-            C.fwd_w[at] = w;
-        }
-        ++o.nf;
-    }
-}
-
-template <class T, int LM>
-__device__ __forceinline__ void force_finish(const Ctx<T>& C, int i, T half_dt, int kick, PairOut<T>& o) {
-    if (o.nn > C.nbr_cap || o.nf > C.nbr_cap) {
-        flag(C.status, ST_CAPACITY);
-        o.nn = min(o.nn, C.nbr_cap);
-        o.nf = min(o.nf, C.nbr_cap);
-    }
-    if (LM == LIST_ALL || LM == LIST_CROSS) C.nbr_n[i] = o.nn;
-    if (LM == LIST_CROSS || LM == LIST_FWD) C.fwd_n[i] = o.nf;
-    vec_t<T> f;
-    f.x = o.fx; f.y = o.fy; f.z = o.fz; f.w = T(0);
-    C.F[i] = f;
-    // each pair is seen from both sides
-    C.upot[i] = T(0.5) * o.u;
-    if (kick) {
-        vec_t<T> pv = C.pB[i];
-        pv.x += half_dt * o.fx; pv.y += half_dt * o.fy; pv.z += half_dt * o.fz;
-        C.pB[i] = pv;
-    }
-}
-
-// Per-particle path on global memory (fallback for tiles whose halo does
-// not fit in shared memory).
-template <class T, int LM>
-__device__ void force_one_global(const Ctx<T>& C, int i, T half_dt, int kick) {
-    const RepInfo& R = C.reps[C.rep_of_slot[i]];
-    const vec_t<T> qi = C.qB[i];
-    const int cc = C.cB[i];
-    const int cx = cell_x(cc), cy = cell_y(cc), cz = cell_z(cc);
-    const int nx = R.nc[0], ny = R.nc[1], nz = R.nc[2];
-    const T lx = cell_len<T>(R, 0), ly = cell_len<T>(R, 1), lz = cell_len<T>(R, 2);
-    const int* bt = brick_tab(C.tab, R);
-    const int bx = __ldg(bt + cx), by = __ldg(bt + nx + cy), bz = __ldg(bt + nx + ny + cz);
-    PairOut<T> o;
-    for (int sg = 0; sg < 27; ++sg) {
-        const int dxc = sg % 3 - 1, dyc = (sg / 3) % 3 - 1, dzc = sg / 9 - 1;
-        int x = cx + dxc, y = cy + dyc, z = cz + dzc;
-        if (R.walls && (z < 0 || z >= nz)) continue;   // nothing beyond a wall
-        x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
-        y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
-        z = z < 0 ? z + nz : (z >= nz ? z - nz : z);
-        const bool cross = __ldg(bt + x) != bx || __ldg(bt + nx + y) != by || __ldg(bt + nx + ny + z) != bz;
-        const int c = cell_index(C.tab, R, x, y, z);
-        const T sx = shift<T>(dxc, lx), sy = shift<T>(dyc, ly), sz = shift<T>(dzc, lz);
-        const int e = C.start[c + 1];
-        for (int j = C.start[c]; j < e; ++j) {
-            if (j == i) continue;
-            const vec_t<T> qj = C.qB[j];
-            const T ddx = (qi.x - qj.x) - sx, ddy = (qi.y - qj.y) - sy, ddz = (qi.z - qj.z) - sz;
-            const T r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-            if (r2 < C.rc2) force_hit<T, LM>(C, i, j, sg > 13 || (sg == 13 && j > i), cross, ddx, ddy, ddz, r2, o);
-        }
-    }
-    force_finish<T, LM>(C, i, half_dt, kick, o);
-}
-
-// Tiled force pass: one block per tile of (up to) 6 x 6 x 6 cells. The tile
-// and its one-cell halo are staged in shared memory in x-fastest halo-cell
-// order (slot order inside a cell), with positions shifted into one frame
-// centred on the tile, so a separation is a plain difference and the three
-// x-cells of each (dy, dz) neighbour row of a particle form one contiguous
-// range. In this layout j is a forward neighbour of i (later segment, or
-// same cell and later slot) exactly when its halo index is larger, and the
-// rows are visited in (segment, slot) order. The lanes of a warp walk the 9
-// rows in step; the candidate loop only records hits (16-bit halo indices)
-// in a per-thread shared buffer, and a second loop over the hits computes
-// forces and lists -- so the costly part runs once per neighbour, not once
-// per candidate of the slowest lane. Halos larger than hcap fall back to the
-// global path.
-constexpr int TILE_THREADS = 256;
-constexpr int TILE_EDGE = 6;       // default tile edge (cells); the autotuner picks 4..8
-constexpr int TILE_EDGE_MAX = 8;
-constexpr int HIT_BUF = 28;        // hits buffered per thread (flushed when full)
-
-// shared bytes before the staged particles, for halo cell capacity hcc
-// ((edge + 2)^3): hstart, gstart, hbrick, rowoff (edge^2 + 1 <= 65), nown, hits
-__host__ __device__ constexpr size_t tile_head_bytes(int hcc) {
-    return ((size_t)(3 * hcc + 1 + 66) * sizeof(int) + (size_t)HIT_BUF * TILE_THREADS * 2 + 31) & ~(size_t)31;
-}
-// shared bytes per staged halo particle: position, global slot, brick, own
-// index with its halo cell
-template <class T>
-__host__ __device__ constexpr size_t tile_per_particle() {
-    return sizeof(vec_t<T>) + 2 * sizeof(int) + sizeof(unsigned int);
-}
-
-// One tile on the calling block. A tile whose halo holds more than hcap
-// particles is appended to `defer` when that list is given (a second launch
-// with a larger capacity takes it), else computed through the global path.
-template <class T, int LM>
-__device__ __forceinline__ void force_tile_run(const Ctx<T>& C, int tile, const int4* __restrict__ tile_org,
-                                               const int4* __restrict__ tile_dim, T half_dt, int kick, int hcap,
-                                               int hcc, int* defer, int* ndefer) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned char* smem = (unsigned char*)(((size_t)smem_raw + 31) & ~(size_t)31);
-    using vec = vec_t<T>;
-    const int4 org = tile_org[tile];
-    const int4 dim = tile_dim[tile];
-    const RepInfo& R = C.reps[org.x];
-    const int HX = dim.x + 2, HY = dim.y + 2, HZ = dim.z + 2;
-    const int HC = HX * HY * HZ;
-    const int nx = R.nc[0], ny = R.nc[1], nz = R.nc[2];
-    // shared layout (sized for HC <= hcc = (edge + 2)^3):
-    //   hstart[hcc+1] gstart[hcc] hbrick[hcc] rowoff[65] nown | hits[HIT_BUF][TILE_THREADS] (u16) |
-    //   q[hcap] glob[hcap] brick[hcap] own[hcap] (u32: halo index | halo cell << 16)
-    int* hstart = (int*)smem;
-    int* gstart = hstart + hcc + 1;
-    int* hbrick = gstart + hcc;
-    int* rowoff = hbrick + hcc;
-    int* nown = rowoff + 65;
-    unsigned short* hits = (unsigned short*)(nown + 1);
-    vec* hq = (vec*)(smem + tile_head_bytes(hcc));
-    int* hglob = (int*)(hq + hcap);
-    int* hbr = hglob + hcap;
-    unsigned int* own = (unsigned int*)(hbr + hcap);   // halo index | halo cell << 16
-    const int* bt = brick_tab(C.tab, R);
-    // 1. halo cells: global start, count, brick (two cells per thread at a
-    //    time, their loads issued together)
-    for (int h0 = threadIdx.x; h0 < HC; h0 += 2 * blockDim.x) {
-        int xs[2], ys[2], zs[2], cs[2];
-        bool use[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int h = h0 + u * (int)blockDim.x;
-            const int hx = h % HX, hy = (h / HX) % HY, hz = h / (HX * HY);
-            int x = org.y + hx - 1, y = org.z + hy - 1, z = org.w + hz - 1;
-            use[u] = h < HC && !(R.walls && (z < 0 || z >= nz));   // beyond a wall: an empty halo cell
-            x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
-            y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
-            z = z < 0 ? z + nz : (z >= nz ? z - nz : z);
-            xs[u] = x; ys[u] = y; zs[u] = z;
-            cs[u] = use[u] ? cell_index(C.tab, R, x, y, z) : 0;
-        }
-        int a[2] = {0, 0}, b[2] = {0, 0}, br[2] = {-1, -1};
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-            if (use[u]) {
-                a[u] = C.start[cs[u]];
-                b[u] = C.start[cs[u] + 1];
-                br[u] = __ldg(bt + xs[u]) | (__ldg(bt + nx + ys[u]) << 10) | (__ldg(bt + nx + ny + zs[u]) << 20);
-            }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int h = h0 + u * (int)blockDim.x;
-            if (h < HC) {
-                gstart[h] = a[u];
-                hstart[h] = b[u] - a[u];
-                hbrick[h] = br[u];
-            }
-        }
-    }
-    __syncthreads();
-    // 2. exclusive scan of the halo counts (a run of up to 4 per thread, HC <= 1000)
-    {
-        __shared__ int sh[32];
-        const int per = (HC + TILE_THREADS - 1) / TILE_THREADS;
-        const int h0 = threadIdx.x * per;
-        int v[4] = {0, 0, 0, 0}, run = 0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (u < per && h0 + u < HC) {
-                v[u] = hstart[h0 + u];
-                run += v[u];
-            }
-        int total;
-        int ex = block_exclusive_scan(run, sh, total);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (u < per && h0 + u < HC) {
-                hstart[h0 + u] = ex;
-                ex += v[u];
-            }
-        if (threadIdx.x == 0) hstart[HC] = total;
-    }
-    __syncthreads();
-    const int H = hstart[HC];
-    const bool staged = H <= hcap;
-    const T lx = cell_len<T>(R, 0), ly = cell_len<T>(R, 1), lz = cell_len<T>(R, 2);
-    // 3. stage the halo particles (tile frame); 4. own-row offsets
-    if (staged) {
-        const int cxh = HX / 2, cyh = HY / 2, czh = HZ / 2;
-        for (int h = threadIdx.x; h < HC; h += blockDim.x) {
-            const int b = hstart[h], n = hstart[h + 1] - b, g = gstart[h];
-            const int hx = h % HX, hy = (h / HX) % HY, hz = h / (HX * HY);
-            const T ox = (T)(hx - cxh) * lx, oy = (T)(hy - cyh) * ly, oz = (T)(hz - czh) * lz;
-            const int br = hbrick[h];
-            // four loads in flight at a time (a cell holds ~3 particles)
-            for (int k0 = 0; k0 < n; k0 += 4) {
-                vec qv[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (k0 + u < n) qv[u] = C.qB[g + k0 + u];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (k0 + u < n) {
-                        const int k = k0 + u;
-                        qv[u].x += ox; qv[u].y += oy; qv[u].z += oz;
-                        hq[b + k] = qv[u];
-                        hglob[b + k] = g + k;
-                        hbr[b + k] = br;
-                    }
-            }
-        }
-    }
-    const int nrow = dim.y * dim.z;   // <= 64: a row per thread of the first two warps
-    {
-        __shared__ int s_w0;
-        const int r = threadIdx.x;
-        int v = 0;
-        if (r < nrow) {
-            const int h = ((r / dim.y + 1) * HY + (r % dim.y + 1)) * HX;
-            v = hstart[h + dim.x + 1] - hstart[h + 1];
-        }
-        int x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if ((r & 31) >= o) x += y;
-        }
-        if (r == 31) s_w0 = x;
-        __syncthreads();
-        if (r < nrow) {
-            const int incl = x + (r >= 32 ? s_w0 : 0);
-            rowoff[r] = incl - v;
-            if (r == nrow - 1) {
-                rowoff[nrow] = incl;
-                *nown = incl;
-            }
-        }
-    }
-    __syncthreads();
-    if (!staged) {
-        if (defer) {
-            if (threadIdx.x == 0) defer[atomicAdd(ndefer, 1)] = tile;
-            return;
-        }
-        // fallback: own particles through the global path
-        for (int r = threadIdx.x; r < nrow; r += blockDim.x) {
-            const int h = ((r / dim.y + 1) * HY + (r % dim.y + 1)) * HX;
-            for (int hc = h + 1; hc <= h + dim.x; ++hc) {
-                const int g = gstart[hc], n = hstart[hc + 1] - hstart[hc];
-                for (int k = 0; k < n; ++k) force_one_global<T, LM>(C, g + k, half_dt, kick);
-            }
-        }
-        return;
-    }
-    // own particles in row order, a thread per own cell
-    for (int rc = threadIdx.x; rc < nrow * dim.x; rc += blockDim.x) {
-        const int r = rc / dim.x, cx = rc - r * dim.x;
-        const int h = ((r / dim.y + 1) * HY + (r % dim.y + 1)) * HX;
-        const int b = hstart[h + 1], k1 = hstart[h + cx + 2];
-        const unsigned int cell = (unsigned int)(h + cx + 1) << 16;
-        for (int k = hstart[h + cx + 1]; k < k1; ++k) own[rowoff[r] + (k - b)] = (unsigned int)k | cell;
-    }
-    __syncthreads();
-    // 5. each own particle: rows in step, hits recorded, then processed
-    const int no = *nown;
-    unsigned short* myhits = hits + threadIdx.x;
-    for (int k0 = 0; k0 < no; k0 += blockDim.x) {
-        const int k = k0 + threadIdx.x;
-        const bool act = k < no;
-        const unsigned int ow = act ? own[k] : 0u;
-        const int hi = (int)(ow & 0xffffu);
-        const vec qi = hq[hi];
-        const int i = hglob[hi];
-        const int mybrick = hbr[hi];
-        // i's halo cell, stored beside its halo index
-        const int hc = (int)(ow >> 16);
-        PairOut<T> o;
-        int nh = 0;
-        auto flush = [&]() {
-            for (int u = 0; u < nh; ++u) {
-                const int hj = myhits[u * TILE_THREADS];
-                const vec qj = hq[hj];
-                const T ddx = qi.x - qj.x, ddy = qi.y - qj.y, ddz = qi.z - qj.z;
-                const T r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-                force_hit<T, LM>(C, i, hglob[hj], hj > hi, hbr[hj] != mybrick, ddx, ddy, ddz, r2, o);
-            }
-            nh = 0;
-        };
-        auto near = [&](int j) {
-            const vec qj = hq[j];
-            const T ddx = qi.x - qj.x, ddy = qi.y - qj.y, ddz = qi.z - qj.z;
-            return ddx * ddx + ddy * ddy + ddz * ddz < C.rc2 && j != hi;
-        };
-        for (int row = 0; row < 9; ++row) {
-            const int base = hc + (row / 3 - 1) * HX * HY + (row % 3 - 1) * HX - 1;
-            const int je = act ? hstart[base + 3] : 0;
-            int j = act ? hstart[base] : 0;
-            // four independent candidates per pass; every candidate is
-            // written to the next free buffer slot and the slot kept only on
-            // a hit (no branch per hit), so hits stay in order
-            for (; j + 4 <= je; j += 4) {
-                if (nh > HIT_BUF - 4) flush();
-                const bool h0 = near(j), h1 = near(j + 1), h2 = near(j + 2), h3 = near(j + 3);
-                myhits[nh * TILE_THREADS] = (unsigned short)j;
-                nh += h0;
-                myhits[nh * TILE_THREADS] = (unsigned short)(j + 1);
-                nh += h1;
-                myhits[nh * TILE_THREADS] = (unsigned short)(j + 2);
-                nh += h2;
-                myhits[nh * TILE_THREADS] = (unsigned short)(j + 3);
-                nh += h3;
-            }
-            for (; j < je; ++j) {
-                if (nh == HIT_BUF) flush();
-                myhits[nh * TILE_THREADS] = (unsigned short)j;
-                nh += near(j);
-            }
-        }
-        flush();
-        if (act) force_finish<T, LM>(C, i, half_dt, kick, o);
-    }
-}
-
-template <class T, int LM>
-__global__ void __launch_bounds__(TILE_THREADS) k_force_tile(Ctx<T> C, const int4* __restrict__ tile_org,
-                                                             const int4* __restrict__ tile_dim, T half_dt,
-                                                             int kick, int hcap, int hcc, int* defer,
-                                                             int* ndefer) {
-    force_tile_run<T, LM>(C, blockIdx.x, tile_org, tile_dim, half_dt, kick, hcap, hcc, defer, ndefer);
-}
-
-// The deferred tiles (dense regions), persistent blocks with a larger halo
-// capacity; a tile beyond even that takes the global path.
-template <class T, int LM>
-__global__ void __launch_bounds__(TILE_THREADS) k_force_tile_dense(Ctx<T> C, const int4* __restrict__ tile_org,
-                                                                   const int4* __restrict__ tile_dim, T half_dt,
-                                                                   int kick, int hcap, int hcc,
-                                                                   const int* __restrict__ defer,
-                                                                   const int* __restrict__ ndefer) {
-    const int n = *ndefer;
-    for (int u = blockIdx.x; u < n; u += gridDim.x) {
-        force_tile_run<T, LM>(C, defer[u], tile_org, tile_dim, half_dt, kick, hcap, hcc, nullptr, nullptr);
-        __syncthreads();
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -921,8 +572,9 @@ __device__ __forceinline__ T warp_owner_sum(const WarpEntries& W, int f0, int ow
 template <class T>
 __device__ __forceinline__ T3<T> ser_dp(const Ctx<T>& C, int i, int k, uint32_t step, T dt, T sdt,
                                         const vec_t<T>& pi, uint32_t idi, int rep) {
-    const int j = C.nbr_j[(size_t)k * C.N + i];
-    const T w = C.nbr_w[(size_t)k * C.N + i];
+    const ListEnt<T> en = C.nbr[(size_t)k * C.N + i];
+    const int j = en.j;
+    const T w = en.w;
     const vec_t<T> pj = C.pB[j];
     const T3<T> G = pair_gauss<T>(C.seed, step, (uint32_t)rep, idi, C.idB[j]);
     const T A = -(C.sig2_4 * (pi.w + pj.w)) * (w * w) * dt;
@@ -1023,7 +675,7 @@ __global__ void k_ser_sweep2(Ctx<T> C, T dt, T sqrt_dt) {
             const int io = base + o;
             const vec_t<T> pi = C.pB[io];
             const vec_t<T> dpi = C.dp[io];
-            const int j = C.nbr_j[(size_t)k * C.N + io];
+            const int j = C.nbr[(size_t)k * C.N + io].j;
             const vec_t<T> d = C.fwd_g[(size_t)k * C.N + io];   // delta p_ij of the first sweep
             const vec_t<T> pj = C.pB[j];
             const vec_t<T> dpj = C.dp[j];
@@ -1068,8 +720,9 @@ __global__ void k_sem(Ctx<T> C, T dt, T sqrt_dt) {
     const T sdt = C.sigma * sqrt_dt;
     T ax = 0, ay = 0, az = 0, de = 0;
     for (int k = 0; k < nn; ++k) {
-        const int j = C.nbr_j[(size_t)k * C.N + i];
-        const T w = C.nbr_w[(size_t)k * C.N + i];
+        const ListEnt<T> en = C.nbr[(size_t)k * C.N + i];
+        const int j = en.j;
+        const T w = en.w;
         const vec_t<T> pj = C.pB[j];
         const T chi = w * w;
         const T gam = C.sig2_4 * (pi.w + pj.w);
@@ -1158,10 +811,10 @@ __global__ void k_ssa_gauss(Ctx<T> C) {
             const int so = base + lo;
             const size_t at = (size_t)(f - excl) * C.N + so;
             const size_t row = (size_t)so * cap + (f - excl);
-            const int t = C.fwd_j[at];
-            const T3<T> G = pair_gauss<T>(C.seed, step, (uint32_t)C.rep_of_slot[so], C.idB[so], C.idB[t]);
+            const ListEnt<T> en = C.fwd[at];
+            const T3<T> G = pair_gauss<T>(C.seed, step, (uint32_t)C.rep_of_slot[so], C.idB[so], C.idB[en.j]);
             vec_t<T> g;
-            g.x = G.x; g.y = G.y; g.z = G.z; g.w = C.fwd_w[at];
+            g.x = G.x; g.y = G.y; g.z = G.z; g.w = en.w;
             C.fwd_g[row] = g;
         }
     }
@@ -1237,7 +890,7 @@ __device__ void ssa_chain_plain(const Ctx<T>& C, const RepInfo& R, int b, int e,
         eps_t<T> es = C.eB[s];
         T bs = ps.w;
         for (int m = 0; m < nf; ++m) {
-            const int t = C.fwd_j[(size_t)m * C.N + s];
+            const int t = C.fwd[(size_t)m * C.N + s].j;
             const vec_t<T> g = C.fwd_g[(size_t)s * cap + m];
             vec_t<T> pt = C.pB[t];
             eps_t<T> et = C.eB[t];
@@ -1301,7 +954,7 @@ __device__ __forceinline__ void ssa_cell_chain(const Ctx<T>& C, int c, T dt, T s
     };
     auto load_index = [&](int r, int m, Ent& x) {
         x.s = row_s[r * bdim + tid];
-        x.t = C.fwd_j[(size_t)m * C.N + x.s];
+        x.t = C.fwd[(size_t)m * C.N + x.s].j;
         x.g = C.fwd_g[(size_t)x.s * cap + m];
     };
     auto load_state = [&](Ent& x, int prev_s) {
@@ -1439,7 +1092,7 @@ template <class T>
 __device__ __forceinline__ bool ssa_fetch(const Ctx<T>& C, int& s, int& m, int& nf, int e, SsaEntry<T>& q) {
     if (!ssa_next(C.fwd_n, s, m, nf, e)) return false;
     q.s = s;
-    q.t = __ldg(C.fwd_j + (size_t)m * C.N + s);
+    q.t = __ldg(&C.fwd[(size_t)m * C.N + s].j);
     q.g = C.fwd_g[(size_t)s * C.nbr_cap + m];
     return true;
 }

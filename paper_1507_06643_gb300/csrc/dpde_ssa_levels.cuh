@@ -198,11 +198,10 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
     for (int i = tid; i < nb; i += blockDim.x) L[i] = 0;
     __syncthreads();   // the rows' offsets were written by other threads
     const size_t N = (size_t)C.N;
-    const int* fj = C.fwd_j + sb;   // entry m of local particle i at fj[m N + i]
-    const T* fw = C.fwd_w + sb;
+    const ListEnt<T>* fe = C.fwd + sb;   // entry m of local particle i at fe[m N + i]
     // 2. partner slots, local
     ssa_rows_mmajor(
-        nb, rowoff, [&](int i, int m) { return __ldg(fj + (size_t)m * N + i) - sb; },
+        nb, rowoff, [&](int i, int m) { return __ldg(&fe[(size_t)m * N + i].j) - sb; },
         [&](int, int e, int t) {
             if ((unsigned)t >= (unsigned)nb) s_flag = 1;   // never by construction
             ent[e] = (unsigned short)min(max(t, 0), nb - 1);
@@ -318,8 +317,8 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
     ssa_rows_mmajor(
         nb, rowoff,
         [&](int i, int m) {
-            const size_t at = (size_t)m * N + i;
-            return TW{__ldg(fj + at) - sb, __ldg(fw + at)};
+            const ListEnt<T> en = fe[(size_t)m * N + i];
+            return TW{en.j - sb, en.w};
         },
         [&](int i, int e, const TW& x) {
             const int pos = cnt_add(cnt, ent[e]);
@@ -455,13 +454,14 @@ __device__ void ssa_exec_classes(const Ctx<T>& C, const SsaDomains& D, int d, in
                 T bs = ps.w;
                 const uint32_t ids = C.idB[s];
                 for (int m = 0; m < nf; ++m) {
-                    const int t = C.fwd_j[(size_t)m * N + s];
+                    const ListEnt<T> en = C.fwd[(size_t)m * N + s];
+                    const int t = en.j;
                     const T3<T> G = pair_gauss<T>(C.seed, step, (uint32_t)rep, ids, C.idB[t]);
                     vec_t<T> g;
                     g.x = G.x;
                     g.y = G.y;
                     g.z = G.z;
-                    g.w = C.fwd_w[(size_t)m * N + s];
+                    g.w = en.w;
                     vec_t<T> pt = C.pB[t];
                     eps_t<T> et = C.eB[t];
                     ssa_pair_map(C, R, ps, es, bs, pt, et, g, k2, amp0);
