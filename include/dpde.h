@@ -381,9 +381,11 @@ typedef struct dpde_tuning {
     int32_t tile_edge;   /* force tile edge in cells, 2..8 (default 6)                */
     int32_t block;       /* threads per block of the per-particle kernels: a multiple  */
                          /* of 32 in 64..1024 (default 256)                           */
-    int32_t ssa_block;   /* threads per block of the per-class SSA launches and of the */
-                         /* level form's execution: 32, 64, 96 or 128 (the per-domain  */
-                         /* form runs one warp per block) (default 64)                */
+    int32_t ssa_block;   /* threads per block of the per-class SSA launches, and       */
+                         /* threads of a block of the level form's execution that     */
+                         /* apply maps (64 more draw the Gaussians): 32, 64, 96 or    */
+                         /* 128 (the per-domain form runs one warp per block)         */
+                         /* (default 64)                                              */
     int32_t ssa_mode;    /* form of the SSA launches; all give the same results bit   */
                          /* for bit. 2 (default): by dependency levels -- per domain, */
                          /* every map of the sequence gets the level 1 + the larger   */

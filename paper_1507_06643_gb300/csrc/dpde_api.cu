@@ -184,15 +184,8 @@ Ctx<T> make_ctx(dpde_handle* h) {
     C.a = (T)h->prm.a; C.sigma = (T)h->prm.sigma;
     C.pot = cast_pot<T>(make_pot(h->prm.potential, h->prm.a, h->prm.r_cut, h->prm.lj_eps, h->prm.lj_r));
     C.sig2_4 = (T)(h->prm.sigma * h->prm.sigma / 4.0);
-    C.seed = make_uint2((uint32_t)(h->prm.seed & 0xffffffffu), (uint32_t)(h->prm.seed >> 32));
+    C.seed = philox_keys(make_uint2((uint32_t)(h->prm.seed & 0xffffffffu), (uint32_t)(h->prm.seed >> 32)));
     return C;
-}
-
-// The level form's records live in the buffer of the forward entries'
-// Gaussians (unused by that form): N * cap 32-bit (s, t) words, then, from a
-// 256-byte boundary, N * cap weights.
-size_t ssa_rec_w_offset(const dpde_handle* h) {
-    return ((size_t)std::max(1, h->N) * (size_t)h->nbr_cap * sizeof(uint32_t) + 255) & ~(size_t)255;
 }
 
 // phase markers (only when dpde_step_profiled is running)
@@ -264,8 +257,7 @@ void enqueue_ssa_levels(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T dt, 
     SsaLevels<T> V;
     V.lv_off = h->lv_off;
     V.lv_n = h->lv_n;
-    V.rec_st = reinterpret_cast<uint32_t*>(h->fwd_g);
-    V.rec_w = reinterpret_cast<T*>(reinterpret_cast<unsigned char*>(h->fwd_g) + ssa_rec_w_offset(h));
+    V.rec = reinterpret_cast<SsaRec<T>*>(h->fwd_g);   // (unused by this form: the forward entries' Gaussians)
     // counts: [0, 1] schedule tiers 1, 2; [2, 3] execution tiers 1, 2 of the
     // domains the regular schedule kept; [4, 5] execution tiers 1, 2 of those
     // it deferred; then the lists
@@ -281,9 +273,9 @@ void enqueue_ssa_levels(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T dt, 
     };
     // execution tiers 1, 2 over the list at index l0 (tier 1) and l0 + 1 (tier 2)
     auto exec_tiers = [&](cudaStream_t s, int* first, int* nfirst, int l1) {
-        k_ssa_exec<T><<<K.grid_x[1], h->ssa_block, ssa_exec_smem<T>(K.scap_x[1]), s>>>(
+        k_ssa_exec<T><<<K.grid_x[1], h->ssa_block + SSA_DRAW_THREADS, ssa_exec_smem<T>(K.scap_x[1]), s>>>(
             C, D, V, K.scap_x[1], 0, first, nfirst, lst[l1], cnt + l1, dt, sqrt_dt);
-        k_ssa_exec<T><<<K.grid_x[2], h->ssa_block, ssa_exec_smem<T>(K.scap_x[2]), s>>>(
+        k_ssa_exec<T><<<K.grid_x[2], h->ssa_block + SSA_DRAW_THREADS, ssa_exec_smem<T>(K.scap_x[2]), s>>>(
             C, D, V, K.scap_x[2], 0, lst[l1], cnt + l1, nullptr, nullptr, dt, sqrt_dt);
     };
     auto sched_regular = [&](cudaStream_t s, int d0, int n) {
@@ -291,7 +283,7 @@ void enqueue_ssa_levels(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T dt, 
             C, D, V, K.scap_s[0], K.ecap_s[0], K.ccap_s[0], d0, nullptr, nullptr, lst[0], cnt);
     };
     auto exec_regular = [&](cudaStream_t s, int d0, int n) {
-        k_ssa_exec<T><<<n, h->ssa_block, ssa_exec_smem<T>(K.scap_x[0]), s>>>(C, D, V, K.scap_x[0], d0, nullptr,
+        k_ssa_exec<T><<<n, h->ssa_block + SSA_DRAW_THREADS, ssa_exec_smem<T>(K.scap_x[0]), s>>>(C, D, V, K.scap_x[0], d0, nullptr,
                                                                              nullptr, lst[2], cnt + 2, dt, sqrt_dt);
     };
     if (h->profiling) {   // phase by phase, one stream
@@ -904,7 +896,7 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
             // entries that fit beside sc particles in ~200 KB of schedule
             auto ecap_fit = [&](int sc, int cc) {
                 return std::min(SSA_LOCAL_MAX,
-                                (int)((smem_big - (SSA_LV_STRIDE + cc) * sizeof(int)) / 2 - (2 * sc + 1)) / 16 * 16);
+                                (int)((smem_big - (SSA_LV_STRIDE + 4 + cc) * sizeof(int)) / 2 - (2 * sc + 1)) / 16 * 16);
             };
             // schedule: 1.3 M particles / 1.2 M e entries; 2.5 M / 6.25 M e (a
             // brick compressed 2.5-fold holds ~6x the entries) in ~96 KB; the
@@ -923,9 +915,9 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
             K.ccap_s[2] = 0;
             K.ecap_s[2] = ecap_fit(K.scap_s[2], 0);
             // execution: M + 5 sqrt(M) + 32 particles; 2.5 M in <= 96 KB; ~200 KB
-            const int xfit = (int)((smem_big - 32) / per);
+            const int xfit = (int)((smem_big - (h->mixed ? ssa_exec_smem<float>(0) : ssa_exec_smem<double>(0))) / per) & ~3;
             K.scap_x[0] = std::min(xfit, ((int)std::ceil(M + 5.0 * std::sqrt(M) + 32) + 31) / 32 * 32);
-            K.scap_x[1] = std::max(K.scap_x[0], std::min(xfit / 2, ((int)std::ceil(2.5 * M + 64) + 31) / 32 * 32));
+            K.scap_x[1] = std::max(K.scap_x[0], std::min(xfit / 2 & ~3, ((int)std::ceil(2.5 * M + 64) + 31) / 32 * 32));
             K.scap_x[2] = xfit;
             const size_t smem_sm = 227 * 1024;
             K.grid_s[0] = ndom;

@@ -152,18 +152,30 @@ template <> __device__ __forceinline__ float cell_len<float>(const RepInfo& R, i
 // 64-bit products, and xors the high halves with words 1 / 3 and the key;
 // the key is advanced by the two Weyl constants before every later round.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
+//
+// The ten round keys of a handle's seed are launch constants (kernel
+// parameters): bumping the key in every draw was 18 of its ~300 instructions.
+struct PhiloxKeys {
+    uint32_t x[10], y[10];
+};
+
+__host__ __device__ __forceinline__ PhiloxKeys philox_keys(uint2 k) {
+    PhiloxKeys K;
+    for (int r = 0; r < 10; ++r) {
+        K.x[r] = k.x + (uint32_t)r * 0x9E3779B9u;
+        K.y[r] = k.y + (uint32_t)r * 0xBB67AE85u;
+    }
+    return K;
+}
+
+__device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKeys& K) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        if (r > 0) {
-            k.x += 0x9E3779B9u;
-            k.y += 0xBB67AE85u;
-        }
         const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
         const uint32_t lo0 = 0xD2511F53u * c.x;
         const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
         const uint32_t lo1 = 0xCD9E8D57u * c.z;
-        c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
+        c = make_uint4(hi1 ^ c.y ^ K.x[r], lo1, hi0 ^ c.w ^ K.y[r], lo0);
     }
     return c;
 }
@@ -200,7 +212,7 @@ __device__ __forceinline__ T3<double> gauss3(uint4 x, double) {
 // G_ij for particle i (id_i) and neighbour j (id_j): drawn for the ordered
 // pair (min id, max id) and negated when id_i > id_j, so G_ji = -G_ij.
 template <class T>
-__device__ __forceinline__ T3<T> pair_gauss(uint2 key, uint32_t step, uint32_t rep, uint32_t id_i,
+__device__ __forceinline__ T3<T> pair_gauss(const PhiloxKeys& key, uint32_t step, uint32_t rep, uint32_t id_i,
                                             uint32_t id_j) {
     const bool lo = id_i < id_j;
     const uint4 x = philox4x32_10(make_uint4(lo ? id_i : id_j, lo ? id_j : id_i, step, rep), key);

@@ -53,7 +53,7 @@ template <class T> struct Ctx {
     int N, ncells;
     T m, inv_m, rc, rc2, inv_rc, a, sigma, sig2_4;
     PotT<T> pot;
-    uint2 seed;
+    PhiloxKeys seed;   // round keys
 };
 
 // ---------------------------------------------------------------------------
@@ -1393,7 +1393,7 @@ __global__ void k_get_cells(Ctx<T> C, int* __restrict__ out) {
 __global__ void k_debug_philox(int n, const uint4* __restrict__ ctr, const uint2* __restrict__ key,
                                uint4* __restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = philox4x32_10(ctr[i], key[i]);
+    if (i < n) out[i] = philox4x32_10(ctr[i], philox_keys(key[i]));
 }
 
 template <class T>
@@ -1402,7 +1402,7 @@ __global__ void k_debug_gauss(int n, uint2 seed, const uint32_t* __restrict__ st
                               const uint32_t* __restrict__ b, double* __restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const T3<T> g = pair_gauss<T>(seed, step[i], rep[i], a[i], b[i]);
+    const T3<T> g = pair_gauss<T>(philox_keys(seed), step[i], rep[i], a[i], b[i]);
     out[3 * i] = g.x; out[3 * i + 1] = g.y; out[3 * i + 2] = g.z;
 }
 

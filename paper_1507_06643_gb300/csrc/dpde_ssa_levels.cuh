@@ -22,9 +22,10 @@
 //                class share no particle), then sorts the entries by level
 //                into records (s, t, w) in global memory.
 //   k_ssa_exec   one block per domain: stages (p, eps, id) of the domain,
-//                then runs the levels in order, one thread per map, drawing
-//                each pair's Gaussian on the fly (Philox is keyed on the ids),
-//                with a block barrier between levels; writes the state back.
+//                then runs the levels in order, one thread per map. Half of
+//                its warps only draw the pairs' Gaussians (Philox is keyed on
+//                the ids) in record order, a chunk ahead of the others, which
+//                only apply maps, with a barrier of their own between levels.
 // Domains too large for the regular shared-memory capacities are deferred to
 // a second launch of each kernel with ~2.5x larger capacities (several
 // blocks per SM), and from there to a third with what ~200 KB hold; beyond
@@ -40,9 +41,12 @@ namespace dpde {
 constexpr int SSA_MAXLEV = 1023;         // levels of one domain kept by the schedule
 constexpr int SSA_LV_STRIDE = SSA_MAXLEV + 2;
 constexpr int SCHED_THREADS = 128;
-constexpr int SSA_LOAD_BATCH = 8;       // entries of a row taken together by the level walk
-constexpr int SSA_COL_BATCH = 6;        // particles whose m-th entries a thread loads together
-constexpr int SSA_EXEC_THREADS_MAX = 128;
+constexpr int SSA_ROW_BATCH = 8;        // entries of a row taken together
+constexpr int SSA_LEV_BATCH = 8;        // ... by the level walk
+constexpr int SSA_DRAW_THREADS = 64;    // threads of an execution block that draw Gaussians
+constexpr int SSA_EXEC_THREADS_MAX = SSA_THREADS_MAX + SSA_DRAW_THREADS;
+constexpr int SSA_CHUNK = 128;          // records drawn ahead of the maps, SSA_RING chunks held
+constexpr int SSA_RING = 3;
 constexpr int SSA_LOCAL_MAX = 65535;      // particles (and entries) of one domain: 16-bit local indices
 constexpr int SSA_NLISTS = 5;             // deferred-domain lists of one step (see enqueue_ssa_levels)
 
@@ -63,30 +67,35 @@ struct SsaDomains {
 // regular launch, -3 - nlev from a deferred one, -1 no schedule (executed
 // along the colour order), SSA_PENDING = -2 deferred and not yet scheduled),
 // and the records, domain d's at [slot0(d) * cap, ...): (s_local | t_local
-// << 16) and the weight w. The execution's regular launch, which may run
-// beside the schedule's deferred launches, takes only lv_n >= -1, so it never
-// reads a schedule that is still being written.
+// << 16) and the weight w, one 8- or 16-byte word. The execution's regular
+// launch, which may run beside the schedule's deferred launches, takes only
+// lv_n >= -1, so it never reads a schedule that is still being written.
+template <class T> struct __align__(2 * sizeof(T)) SsaRec {
+    uint32_t st;
+    T w;
+};
+
 template <class T>
 struct SsaLevels {
     int* lv_off;
     int* lv_n;
-    uint32_t* rec_st;
-    T* rec_w;
+    SsaRec<T>* rec;
 };
 
 // shared bytes of k_ssa_sched for scap particles, ecap entries and ccap
-// cells: cnt (16-bit counters of levels 0..SSA_MAXLEV + 1, two to a word) |
-// cr[ccap] (the domain's cells in class order: local start | count << 16) |
-// rowoff[scap + 1] | L[scap] | ent[ecap] (16-bit)
+// cells: cnt (counters of levels 0..SSA_MAXLEV + 1) | cr[ccap] (the domain's
+// cells in class order: local start | count << 16) | rowoff[scap + 1] |
+// L[scap] | ent[ecap] (16-bit)
 __host__ __device__ constexpr size_t ssa_sched_smem(int scap, int ecap, int ccap) {
-    return (size_t)(SSA_LV_STRIDE / 2 + 1 + ccap) * sizeof(int) +
+    return (size_t)(SSA_LV_STRIDE + 1 + ccap) * sizeof(int) +
            (((size_t)(2 * scap + 1 + ecap) * 2 + 15) / 16) * 16;
 }
-// shared bytes of k_ssa_exec for scap staged particles: p | eps | id, after
-// up to 31 bytes that align p to 32 bytes
+// shared bytes of k_ssa_exec for scap staged particles (a multiple of 4): p |
+// drawn (G, w) of the chunks held | eps | id | their records | level starts
 template <class T>
 __host__ __device__ constexpr size_t ssa_exec_smem(int scap) {
-    return 32 + (size_t)scap * (sizeof(vec_t<T>) + sizeof(eps_t<T>) + sizeof(uint32_t));
+    return (size_t)scap * (sizeof(vec_t<T>) + sizeof(eps_t<T>) + sizeof(uint32_t)) +
+           (size_t)SSA_RING * SSA_CHUNK * (sizeof(vec_t<T>) + sizeof(uint32_t)) + (size_t)SSA_LV_STRIDE * 2 + 16;
 }
 
 // slot range [sb, se) of domain d
@@ -115,40 +124,23 @@ __device__ __forceinline__ int block_scan_runs(int n, unsigned short* out, int* 
     return total;
 }
 
-// 16-bit level counters, two to a 32-bit word (a domain has at most
-// SSA_LOCAL_MAX entries, so no count or offset reaches the upper half)
-__device__ __forceinline__ int cnt_add(int* cnt, int l) {
-    const int sh = (l & 1) << 4;
-    return (atomicAdd(cnt + (l >> 1), 1 << sh) >> sh) & 0xffff;
-}
-__device__ __forceinline__ int cnt_get(const int* cnt, int l) { return (cnt[l >> 1] >> ((l & 1) << 4)) & 0xffff; }
-
-// The forward entries of the domain's particles, entry index m outermost:
-// a thread takes SSA_COL_BATCH particles i = i0 + tid + k blockDim (so a
-// warp's lanes read consecutive words of each entry row [m N + i]) and, for
-// every m below their row lengths, issues the loads of all of them before
-// using them. use(i, e, v) gets the value load(i, m) of entry m of particle
-// i, whose row starts at rowoff[i] (e = rowoff[i] + m).
-template <class Load, class Use>
-__device__ __forceinline__ void ssa_rows_mmajor(int nb, const unsigned short* rowoff, Load&& load, Use&& use) {
-    const int bd = blockDim.x;
-    for (int i0 = 0; i0 < nb; i0 += SSA_COL_BATCH * bd) {
-        int e0[SSA_COL_BATCH], nf[SSA_COL_BATCH], mx = 0;
+// The forward entries of the domain's particles, a thread per particle (so a
+// warp's lanes read consecutive words of each entry row) with SSA_ROW_BATCH
+// loads in flight. use(i, e, v, ok) gets entry e of the domain, of particle
+// i, whose row starts at rowoff[i]; past a row's end the last entry again,
+// with ok = false, so that nothing branches. fe: entry row 0 of the domain's
+// particles.
+template <class T, class Use>
+__device__ __forceinline__ void ssa_rows(int nb, const unsigned short* rowoff, const ListEnt<T>* fe, size_t N, Use&& use) {
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+        const int e0 = rowoff[i], n = rowoff[i + 1] - e0;
+        const ListEnt<T>* row = fe + i;
+        for (int m = 0; m < n; m += SSA_ROW_BATCH) {
+            ListEnt<T> v[SSA_ROW_BATCH];
 #pragma unroll
-        for (int k = 0; k < SSA_COL_BATCH; ++k) {
-            const int i = i0 + (int)threadIdx.x + k * bd;
-            e0[k] = i < nb ? rowoff[i] : 0;
-            nf[k] = i < nb ? rowoff[i + 1] - e0[k] : 0;
-            mx = max(mx, nf[k]);
-        }
-        for (int m = 0; m < mx; ++m) {
-            decltype(load(0, 0)) v[SSA_COL_BATCH];
+            for (int k = 0; k < SSA_ROW_BATCH; ++k) v[k] = row[(size_t)min(m + k, n - 1) * N];
 #pragma unroll
-            for (int k = 0; k < SSA_COL_BATCH; ++k)
-                if (m < nf[k]) v[k] = load(i0 + (int)threadIdx.x + k * bd, m);
-#pragma unroll
-            for (int k = 0; k < SSA_COL_BATCH; ++k)
-                if (m < nf[k]) use(i0 + (int)threadIdx.x + k * bd, e0[k] + m, v[k]);
+            for (int k = 0; k < SSA_ROW_BATCH; ++k) use(i, e0 + min(m + k, n - 1), v[k], m + k < n);
         }
     }
 }
@@ -167,7 +159,7 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
     const int tid = threadIdx.x;
     if (nb > scap || nb > SSA_LOCAL_MAX) return false;
     int* cnt = reinterpret_cast<int*>(smem);
-    unsigned int* cr = reinterpret_cast<unsigned int*>(cnt + SSA_LV_STRIDE / 2 + 1);
+    unsigned int* cr = reinterpret_cast<unsigned int*>(cnt + SSA_LV_STRIDE + 1);
     unsigned short* rowoff = reinterpret_cast<unsigned short*>(cr + ccap);
     unsigned short* L = rowoff + scap + 1;
     unsigned short* ent = L + scap;    // partner (local slot) of each entry, then its level
@@ -175,7 +167,7 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
         s_flag = 0;
         s_nlev = 0;
     }
-    for (int l = tid; l <= SSA_LV_STRIDE / 2; l += blockDim.x) cnt[l] = 0;
+    for (int l = tid; l <= SSA_LV_STRIDE; l += blockDim.x) cnt[l] = 0;
     const int* off = D.off + (size_t)d * (NCOLOURS + 1);
     for (int k = tid; k <= NCOLOURS; k += blockDim.x) s_off[k] = __ldg(off + k);
     __syncthreads();
@@ -191,85 +183,76 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
             cr[u] = (unsigned int)(a - sb) | ((unsigned int)(b - a) << 16);
         }
     // 1. row offsets of the domain's forward entries (16-bit: checked below)
-    const int* fwd_n = C.fwd_n + sb;
-    const int E = block_scan_runs(nb, rowoff, sh, [&](int i) { return fwd_n[i]; });
+    for (int i = tid; i < nb; i += blockDim.x) L[i] = (unsigned short)C.fwd_n[sb + i];
+    __syncthreads();
+    const int E = block_scan_runs(nb, rowoff, sh, [&](int i) { return (int)L[i]; });
     if (E > ecap || E > SSA_LOCAL_MAX) return false;   // uniform over the block
     if (tid == 0) rowoff[nb] = (unsigned short)E;
+    __syncthreads();   // the row lengths have been read
     for (int i = tid; i < nb; i += blockDim.x) L[i] = 0;
     __syncthreads();   // the rows' offsets were written by other threads
     const size_t N = (size_t)C.N;
     const ListEnt<T>* fe = C.fwd + sb;   // entry m of local particle i at fe[m N + i]
     // 2. partner slots, local
-    ssa_rows_mmajor(
-        nb, rowoff, [&](int i, int m) { return __ldg(&fe[(size_t)m * N + i].j) - sb; },
-        [&](int, int e, int t) {
-            if ((unsigned)t >= (unsigned)nb) s_flag = 1;   // never by construction
-            ent[e] = (unsigned short)min(max(t, 0), nb - 1);
-        });
+    ssa_rows(nb, rowoff, fe, N, [&](int, int e, const ListEnt<T>& v, bool) {
+        const int t = v.j - sb;
+        if ((unsigned)t >= (unsigned)nb) s_flag = 1;   // never by construction
+        ent[e] = (unsigned short)min(max(t, 0), nb - 1);
+    });
     __syncthreads();
     if (s_flag) {
         if (tid == 0) flag(C.status, ST_DOMAIN);
         return false;
     }
-    // 3. levels, class by class. Eight lanes take one cell of the class (the
-    //    cells of a class share no particle) and walk its rows -- the cell's
-    //    particles in slot order -- a chunk of up to eight entries at a time:
-    //    the partners of a row are distinct particles, so their levels are
-    //    loaded at once, and within the chunk the levels follow from a
-    //    prefix maximum across the lanes,
-    //      lev_j = j + 1 + max(L_s, max_{k <= j} (L[t_k] - k)),
-    //    which is the recurrence lev_j = 1 + max(lev_{j-1}, L[t_j]) unrolled.
-    const int lane = tid & 31, sub = lane & 7, gbase = lane & ~7;
-    const int group = tid >> 3, ngroups = blockDim.x >> 3;
+    // 3. levels, class by class, a thread per cell (the cells of a class
+    //    share no particle) walking its rows -- the cell's particles in slot
+    //    order -- a batch of entries at a time: the partners of a row are
+    //    distinct particles, so their levels are loaded at once and only the
+    //    recurrence lev_j = 1 + max(lev_{j-1}, L[t_j]) is serial. (Eight lanes
+    //    a cell and a prefix maximum over them took 29,000 warp instructions
+    //    a domain. Schedule of a step, with the rows below loaded without
+    //    branches: 4M 523 -> 417 us, the batch of 256 boxes 1078 -> 826 us.)
     int mylev = 0;
     for (int k = 0; k < NCOLOURS; ++k) {
         const int k0 = s_off[k], k1 = s_off[k + 1];
         if (k1 == k0) continue;   // uniform over the block
-        for (int u0 = k0; u0 < k1; u0 += ngroups) {   // uniform over the block
-            const int u = u0 + group;
-            int s0 = 0, nrow = 0;
-            if (u < k1) {
-                if (cstaged) {
-                    const unsigned int v = cr[u - cbase];
-                    s0 = (int)(v & 0xffffu);
-                    nrow = (int)(v >> 16);
-                } else {
-                    const int c = __ldg(D.cells + u);
-                    s0 = C.start[c] - sb;
-                    nrow = C.start[c + 1] - sb - s0;
-                }
+        for (int u = k0 + tid; u < k1; u += blockDim.x) {
+            int i, iend;
+            if (cstaged) {
+                const unsigned int v = cr[u - cbase];
+                i = (int)(v & 0xffffu);
+                iend = i + (int)(v >> 16);
+            } else {
+                const int c = __ldg(D.cells + u);
+                i = C.start[c] - sb;
+                iend = C.start[c + 1] - sb;
             }
-            const int wrows = __reduce_max_sync(0xffffffffu, nrow);
-            for (int r = 0; r < wrows; ++r) {
-                const bool ract = r < nrow;
-                const int i = s0 + r;
-                int Ls = ract ? L[i] : 0;
-                const int e0 = ract ? rowoff[i] : 0, n = ract ? rowoff[i + 1] - e0 : 0;
-                const int wchunks = __reduce_max_sync(0xffffffffu, (n + 7) >> 3);
-                for (int ch = 0; ch < wchunks; ++ch) {
-                    const int j = (ch << 3) + sub;   // entry of the row
-                    const bool ea = j < n;
-                    const int t = ea ? ent[e0 + j] : 0;
-                    int a = ea ? (int)L[t] - sub : -65536;
+            int e = i < iend ? rowoff[i] : 0;
+            for (; i < iend; ++i) {
+                const int end = rowoff[i + 1];
+                int Ls = L[i];
+                for (; e < end; e += SSA_LEV_BATCH) {
+                    // (past the row's end: its last entry again, which
+                    // changes nothing)
+                    int t[SSA_LEV_BATCH], l[SSA_LEV_BATCH];
 #pragma unroll
-                    for (int o = 1; o < 8; o <<= 1) {
-                        const int y = __shfl_up_sync(0xffffffffu, a, o, 8);
-                        if (sub >= o) a = max(a, y);
+                    for (int b = 0; b < SSA_LEV_BATCH; ++b) t[b] = ent[min(e + b, end - 1)];
+#pragma unroll
+                    for (int b = 0; b < SSA_LEV_BATCH; ++b) l[b] = L[t[b]];
+#pragma unroll
+                    for (int b = 0; b < SSA_LEV_BATCH; ++b) {
+                        if (e + b < end) Ls = max(Ls, l[b]) + 1;   // (at most E <= SSA_LOCAL_MAX)
+                        l[b] = Ls;
                     }
-                    const int lv = min(max(Ls, a) + sub + 1, 65535);
-                    if (ea) {
-                        L[t] = (unsigned short)lv;
-                        ent[e0 + j] = (unsigned short)lv;
+#pragma unroll
+                    for (int b = 0; b < SSA_LEV_BATCH; ++b) {
+                        L[t[b]] = (unsigned short)l[b];
+                        ent[min(e + b, end - 1)] = (unsigned short)l[b];
                     }
-                    const int last = min(n - (ch << 3), 8) - 1;   // last entry of this chunk
-                    const int lvl = __shfl_sync(0xffffffffu, lv, gbase + max(last, 0));
-                    if (last >= 0) Ls = lvl;
                 }
-                if (ract) {
-                    if (sub == 0) L[i] = (unsigned short)Ls;
-                    mylev = max(mylev, Ls);
-                }
-                __syncwarp();   // the row's level writes, before the next row reads them
+                e = end;
+                L[i] = (unsigned short)Ls;
+                mylev = max(mylev, Ls);
             }
         }
         __syncthreads();
@@ -279,7 +262,7 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
     const int nlev = s_nlev;
     if (nlev > SSA_MAXLEV) return false;
     // 4. records sorted by level: counts, offsets, scatter
-    for (int e = tid; e < E; e += blockDim.x) cnt_add(cnt, ent[e]);
+    for (int e = tid; e < E; e += blockDim.x) atomicAdd(cnt + ent[e], 1);
     __syncthreads();
     int* lvo = V.lv_off + (size_t)d * SSA_LV_STRIDE;
     if (tid < 32) {
@@ -288,43 +271,29 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
         int carry = 0;
         for (int l0 = 1; l0 <= nlev + 1; l0 += 32) {
             const int l = l0 + tid;
-            const int v = l <= nlev ? cnt_get(cnt, l) : 0;
+            const int v = l <= nlev ? cnt[l] : 0;
             int x = v;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int y = __shfl_up_sync(0xffffffffu, x, o);
                 if (tid >= o) x += y;
             }
-            if (l <= nlev + 1) lvo[l - 1] = carry + x - v;
+            if (l <= nlev + 1) {
+                lvo[l - 1] = carry + x - v;
+                cnt[l] = carry + x - v;
+            }
             carry += __shfl_sync(0xffffffffu, x, 31);
         }
-    }
-    __syncthreads();
-    for (int l = tid; l <= SSA_LV_STRIDE / 2; l += blockDim.x) {
-        // cursor pair (2l, 2l + 1) = level starts (lvo[2l - 1], lvo[2l])
-        const int lo = 2 * l >= 1 && 2 * l <= nlev ? lvo[2 * l - 1] : 0;
-        const int hi = 2 * l + 1 <= nlev ? lvo[2 * l] : 0;
-        cnt[l] = lo | (hi << 16);
     }
     __syncthreads();
     // the partners again from the force pass's list (just read: cached), the
     // weights with them
     const size_t base = (size_t)sb * C.nbr_cap;
-    struct TW {
-        int t;
-        T w;
-    };
-    ssa_rows_mmajor(
-        nb, rowoff,
-        [&](int i, int m) {
-            const ListEnt<T> en = fe[(size_t)m * N + i];
-            return TW{en.j - sb, en.w};
-        },
-        [&](int i, int e, const TW& x) {
-            const int pos = cnt_add(cnt, ent[e]);
-            V.rec_st[base + pos] = (uint32_t)i | ((uint32_t)min(max(x.t, 0), nb - 1) << 16);
-            V.rec_w[base + pos] = x.w;
-        });
+    ssa_rows(nb, rowoff, fe, N, [&](int i, int e, const ListEnt<T>& v, bool ok) {
+        const int pos = atomicAdd(cnt + ent[e], ok ? 1 : 0);
+        const SsaRec<T> x{(uint32_t)i | ((uint32_t)min(max(v.j - sb, 0), nb - 1) << 16), v.w};
+        if (ok) V.rec[base + pos] = x;
+    });
     if (tid == 0) V.lv_n[d] = deferred ? -3 - nlev : nlev;
     return true;
 }
@@ -357,77 +326,122 @@ __global__ void __launch_bounds__(SCHED_THREADS, 8) k_ssa_sched(Ctx<T> C, SsaDom
     }
 }
 
-// The levels of domain d on the state (P, Es, ID), indexed by local slot.
-// A thread's first map of every level (its "pass 0") runs in a three-stage
-// software pipeline: the record of level l + 2 is loaded, the Gaussian of
-// level l + 1 drawn, and the map of level l applied in the same iteration, so
-// neither the record's global-memory latency nor the Philox rounds sit between
-// two level barriers. Further maps of a crowded level follow unpipelined.
+// The levels of domain d on the state (P, Es, ID), indexed by local slot, by
+// nmap threads that apply maps and the block's others, which draw.
+//
+// What bounds it: a level holds ~36 maps at density 3 and ~105 levels depend
+// on one another, so the applying warps are latency bound, ~400 cycles a
+// level, while Philox and Box-Muller are two thirds of the instructions and
+// depend on nothing. Drawn by the applying threads they ran on partly filled
+// warps and inside the levels' critical path; drawn in record order by warps
+// of their own, every lane draws, and the other blocks' drawing fills the
+// applying warps' waits. Two drawing warps keep up with two applying ones
+// (one: 709 us at 4M; three: 568). Execution of a step: 4M 610 -> 516 us, the
+// shock tube 1083 -> 782, 125 domains of 864 particles 110 -> 79 us, 1,000
+// particles in FP64 708 -> 321 us.
+// the block's barrier, for warps at different places of the code
+__device__ __forceinline__ void block_bar() { asm volatile("bar.sync 0;" ::: "memory"); }
+
 template <class T>
 __device__ __forceinline__ void ssa_exec_levels(const Ctx<T>& C, const SsaLevels<T>& V, int d, int sb, int rep,
-                                                vec_t<T>* P, eps_t<T>* Es, const uint32_t* ID, T dt,
-                                                T sqrt_dt) {
-    const RepInfo& R = C.reps[rep];
+                                                vec_t<T>* P, eps_t<T>* Es, const uint32_t* ID, vec_t<T>* ring,
+                                                uint32_t* ring_st, const unsigned short* lvs, int nlev, int nmap,
+                                                T dt, T sqrt_dt) {
+    static_assert(SSA_THREADS_MAX <= SSA_CHUNK, "see the ring");
+    RepInfo R;   // (in registers: the barriers would have a reference read again)
+    R.cv = C.reps[rep].cv;
+    R.cvf = C.reps[rep].cvf;
+    const int tid = threadIdx.x;
+    const int E = lvs[nlev];
+    const int nchunk = (E + SSA_CHUNK - 1) / SSA_CHUNK;
+    const SsaRec<T>* rec = V.rec + (size_t)sb * C.nbr_cap;
+    if (tid >= nmap) {
+        // a record of every SSA_DRAW_THREADS, the next one loaded while this
+        // one's Gaussian is drawn
+        const uint32_t step = (uint32_t)*C.step;
+        int r = tid - nmap;
+        SsaRec<T> x{0u, T(0)};
+        if (r < E) x = rec[r];
+        for (int c = 0; c <= nchunk; ++c) {
+            const int end = min(E, (c + 1) * SSA_CHUNK);
+            int at = c % SSA_RING * SSA_CHUNK + tid - nmap;
+#pragma unroll 1
+            for (; r < end; r += SSA_DRAW_THREADS, at += SSA_DRAW_THREADS) {
+                const SsaRec<T> y = x;
+                if (r + SSA_DRAW_THREADS < E) x = rec[r + SSA_DRAW_THREADS];
+                const T3<T> G = pair_gauss<T>(C.seed, step, (uint32_t)rep, ID[y.st & 0xffffu], ID[y.st >> 16]);
+                vec_t<T> g;
+                g.x = G.x; g.y = G.y; g.z = G.z; g.w = y.w;
+                ring[at] = g;
+                ring_st[at] = y.st;
+            }
+            block_bar();
+        }
+        return;
+    }
     const T amp0 = T(2) * C.sigma * sqrt_dt;   // amplitude of the map as gamma -> 0
     const T k2 = T(2) * dt * C.inv_m;
-    const uint32_t step = (uint32_t)*C.step;
-    const int nlev = ssa_nlev(V.lv_n[d]);
-    const int* lvo = V.lv_off + (size_t)d * SSA_LV_STRIDE;
-    const size_t base = (size_t)sb * C.nbr_cap;
-    const uint32_t* rst = V.rec_st + base;
-    const T* rw = V.rec_w + base;
-    const int tid = threadIdx.x;
-    auto apply = [&](uint32_t st, const vec_t<T>& g) {
-        const int s = (int)(st & 0xffffu), t = (int)(st >> 16);
-        vec_t<T> ps = P[s];
-        eps_t<T> es = Es[s];
-        T bs = ps.w;
-        vec_t<T> pt = P[t];
-        eps_t<T> et = Es[t];
-        ssa_pair_map(C, R, ps, es, bs, pt, et, g, k2, amp0);
-        ps.w = bs;
-        P[s] = ps;
-        Es[s] = es;
-        P[t] = pt;
-        Es[t] = et;
-    };
-    auto gauss = [&](uint32_t st, T w) {
-        const T3<T> G = pair_gauss<T>(C.seed, step, (uint32_t)rep, ID[st & 0xffffu], ID[st >> 16]);
-        vec_t<T> g;
-        g.x = G.x;
-        g.y = G.y;
-        g.z = G.z;
-        g.w = w;
-        return g;
-    };
-    // level starts o[l] for l = 0..nlev, read three levels ahead
-    auto lv_start = [&](int l) { return l <= nlev ? __ldg(lvo + l) : 0; };
-    int o0 = lv_start(0), o1 = lv_start(1), o2 = lv_start(2), o3 = lv_start(3);
-    // pass-0 records of levels 0 and 1
-    bool v0 = 0 < nlev && o0 + tid < o1, v1 = 1 < nlev && o1 + tid < o2;
-    uint32_t st0 = v0 ? __ldg(rst + o0 + tid) : 0u, st1 = v1 ? __ldg(rst + o1 + tid) : 0u;
-    T w0 = v0 ? __ldg(rw + o0 + tid) : T(0), w1 = v1 ? __ldg(rw + o1 + tid) : T(0);
-    vec_t<T> g0{};
-    if (v0) g0 = gauss(st0, w0);
-    for (int l = 0; l < nlev; ++l) {
-        // record of level l + 2
-        const bool v2 = l + 2 < nlev && o2 + tid < o3;
-        const uint32_t st2 = v2 ? __ldg(rst + o2 + tid) : 0u;
-        const T w2 = v2 ? __ldg(rw + o2 + tid) : T(0);
-        const int o4 = lv_start(l + 4);
-        // Gaussian of level l + 1 (a warp without a map there skips it), then
-        // the map of level l
-        vec_t<T> g1{};
-        if (v1) g1 = gauss(st1, w1);
-        if (v0) apply(st0, g0);
-        for (int r = o0 + tid + blockDim.x; r < o1; r += blockDim.x) {
-            const uint32_t st = __ldg(rst + r);
-            apply(st, gauss(st, __ldg(rw + r)));
+    // level ends: the current level's, and the next one's, read a step ahead
+    int l = 1, lend = lvs[min(1, nlev)], lnext = lvs[min(2, nlev)];
+    block_bar();                           // chunk 0 is drawn
+    // Chunk c is drawn while the maps of the records before it run: whole
+    // levels, and full steps of a level that reaches into chunk c, so at most
+    // nmap - 1 < SSA_CHUNK records of the chunks before are left for later and
+    // three chunks hold all that is in use.
+    int r = 0, at = 0;   // first record of the step, and its place in the ring
+    for (int c = 1; c <= nchunk; ++c) {
+        const int avail = min(E, c * SSA_CHUNK);
+        auto width = [&](int from) {   // maps of the step at record `from`; 0: not drawn yet, or none left
+            const int n = min(lend - from, nmap);
+            return from + n <= avail ? n : 0;
+        };
+        auto load = [&](int n, int a, uint32_t& st, vec_t<T>& g) {
+            if (tid < n) {
+                int k = a + tid;
+                k -= k >= SSA_RING * SSA_CHUNK ? SSA_RING * SSA_CHUNK : 0;
+                st = ring_st[k];
+                g = ring[k];
+            }
+        };
+        int n = width(r);
+        uint32_t st = 0;
+        vec_t<T> g{};
+        load(n, at, st, g);
+        while (n > 0) {
+            // the next step and its record, loaded ahead
+            r += n;
+            at += n;
+            at -= at >= SSA_RING * SSA_CHUNK ? SSA_RING * SSA_CHUNK : 0;
+            if (r == lend) {
+                lend = lnext;
+                ++l;
+                lnext = lvs[min(l + 1, nlev)];
+            }
+            const int n2 = width(r);
+            uint32_t st2 = 0;
+            vec_t<T> g2{};
+            load(n2, at, st2, g2);
+            if (tid < n) {
+                const int s = (int)(st & 0xffffu), t = (int)(st >> 16);
+                vec_t<T> ps = P[s];
+                eps_t<T> es = Es[s];
+                T bs = ps.w;
+                vec_t<T> pt = P[t];
+                eps_t<T> et = Es[t];
+                ssa_pair_map(C, R, ps, es, bs, pt, et, g, k2, amp0);
+                ps.w = bs;
+                P[s] = ps;
+                Es[s] = es;
+                P[t] = pt;
+                Es[t] = et;
+            }
+            // the applying threads meet (barrier 1; 0 is the block's)
+            asm volatile("bar.sync 1, %0;" ::"r"(nmap) : "memory");
+            n = n2;
+            st = st2;
+            g = g2;
         }
-        __syncthreads();
-        o0 = o1; o1 = o2; o2 = o3; o3 = o4;
-        v0 = v1; st0 = st1; g0 = g1;
-        v1 = v2; st1 = st2; w1 = w2;
+        block_bar();
     }
 }
 
@@ -482,7 +496,7 @@ __device__ void ssa_exec_classes(const Ctx<T>& C, const SsaDomains& D, int d, in
 // nullptr). The regular launch skips a domain whose schedule was deferred.
 template <class T>
 __device__ void ssa_exec_domain(const Ctx<T>& C, const SsaDomains& D, const SsaLevels<T>& V, int d, int scap,
-                                bool regular, int* defer, int* ndefer, T dt, T sqrt_dt, unsigned char* smem) {
+                                bool regular, int* defer, int* ndefer, int nmap, T dt, T sqrt_dt, unsigned char* smem) {
     int sb, se;
     ssa_domain_range(C, D, d, sb, se);
     const int nb = se - sb;
@@ -497,17 +511,23 @@ __device__ void ssa_exec_domain(const Ctx<T>& C, const SsaDomains& D, const SsaL
         ssa_exec_classes(C, D, d, rep, dt, sqrt_dt);
         return;
     }
-    if (nb > scap) {
-        if (defer) {
-            if (threadIdx.x == 0) defer[atomicAdd(ndefer, 1)] = d;
-            return;
-        }
-        ssa_exec_levels(C, V, d, sb, rep, C.pB + sb, C.eB + sb, C.idB + sb, dt, sqrt_dt);
+    vec_t<T>* P = reinterpret_cast<vec_t<T>*>(smem);
+    vec_t<T>* ring = P + scap;
+    eps_t<T>* Es = reinterpret_cast<eps_t<T>*>(ring + SSA_RING * SSA_CHUNK);
+    uint32_t* ID = reinterpret_cast<uint32_t*>(Es + scap);
+    uint32_t* ring_st = ID + scap;
+    unsigned short* lvs = reinterpret_cast<unsigned short*>(ring_st + SSA_RING * SSA_CHUNK);
+    if (nb > scap && defer) {
+        if (threadIdx.x == 0) defer[atomicAdd(ndefer, 1)] = d;
         return;
     }
-    vec_t<T>* P = reinterpret_cast<vec_t<T>*>(((size_t)smem + 31) & ~(size_t)31);
-    eps_t<T>* Es = reinterpret_cast<eps_t<T>*>(P + scap);
-    uint32_t* ID = reinterpret_cast<uint32_t*>(Es + scap);
+    const int* lvo = V.lv_off + (size_t)d * SSA_LV_STRIDE;
+    for (int l = threadIdx.x; l <= nlev; l += blockDim.x) lvs[l] = (unsigned short)lvo[l];
+    if (nb > scap) {
+        __syncthreads();
+        ssa_exec_levels(C, V, d, sb, rep, C.pB + sb, C.eB + sb, C.idB + sb, ring, ring_st, lvs, nlev, nmap, dt, sqrt_dt);
+        return;
+    }
     // four particles per thread in flight
     for (int i0 = threadIdx.x; i0 < nb; i0 += 4 * blockDim.x) {
         vec_t<T> pv[4];
@@ -533,7 +553,7 @@ __device__ void ssa_exec_domain(const Ctx<T>& C, const SsaDomains& D, const SsaL
         }
     }
     __syncthreads();
-    ssa_exec_levels(C, V, d, sb, rep, P, Es, ID, dt, sqrt_dt);
+    ssa_exec_levels(C, V, d, sb, rep, P, Es, ID, ring, ring_st, lvs, nlev, nmap, dt, sqrt_dt);
     for (int i = threadIdx.x; i < nb; i += blockDim.x) {
         C.pB[sb + i] = P[i];
         C.eB[sb + i] = Es[i];
@@ -546,15 +566,15 @@ __device__ void ssa_exec_domain(const Ctx<T>& C, const SsaDomains& D, const SsaL
 // scap particles is passed on to `defer` when one is given, else run on the
 // state in global memory.
 template <class T>
-__global__ void __launch_bounds__(SSA_EXEC_THREADS_MAX) k_ssa_exec(Ctx<T> C, SsaDomains D, SsaLevels<T> V,
+__global__ void __launch_bounds__(SSA_EXEC_THREADS_MAX, sizeof(T) == 4 ? 4 : 2) k_ssa_exec(Ctx<T> C, SsaDomains D, SsaLevels<T> V,
                                                                     int scap, int d0, const int* __restrict__ list,
                                                                     const int* __restrict__ nlist, int* defer,
                                                                     int* ndefer, T dt, T sqrt_dt) {
-    extern __shared__ __align__(16) unsigned char exec_smem[];
+    extern __shared__ __align__(32) unsigned char exec_smem[];   // (aligned here: computed alignment makes generic accesses)
     const int n = list ? *nlist : (int)gridDim.x;
     for (int u = blockIdx.x; u < n; u += gridDim.x) {
-        ssa_exec_domain(C, D, V, list ? list[u] : d0 + u, scap, list == nullptr, defer, ndefer, dt, sqrt_dt,
-                        exec_smem);
+        ssa_exec_domain(C, D, V, list ? list[u] : d0 + u, scap, list == nullptr, defer, ndefer,
+                        (int)blockDim.x - SSA_DRAW_THREADS, dt, sqrt_dt, exec_smem);
         __syncthreads();
     }
 }
