@@ -44,6 +44,7 @@ struct GraphKey {
 
 }  // namespace
 
+constexpr size_t FORCE_SMEM_MAX = 200 * 1024;   // dynamic shared memory of a force block, at most
 constexpr size_t SSA_ALONE_SMEM = 116 * 1024;   // one such block per SM
 constexpr int STATE_CHUNKS = 4;   // chunks of a host <-> device state transfer
 
@@ -218,20 +219,28 @@ void enqueue_sort(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T half_dt, T
 
 template <class T>
 void enqueue_force(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T half_dt, int kick, int list) {
+    // the observables' pass forms its pairs cell by cell: float positions for
+    // the filter beside the cell offsets
+    ForceShape S0 = h->tile_shape, S1 = h->tile_shape_dense;
+    if (list == LIST_OBS) {
+        S0.wide = S1.wide = 1;
+        while (S0.hcap > 64 && force_smem<T>(S0, h->tile_warps) > FORCE_SMEM_MAX) S0.hcap = (S0.hcap * 15 / 16) & ~3;
+        while (S1.hcap > 64 && force_smem<T>(S1, h->tile_warps_dense) > FORCE_SMEM_MAX) S1.hcap = (S1.hcap * 15 / 16) & ~3;
+    }
     const dim3 g(h->ntiles), blk(32 * h->tile_warps), gd(h->ndense_blocks), bd(32 * h->tile_warps_dense);
-    const size_t sm = force_smem<T>(h->tile_shape, h->tile_warps),
-                 smd = force_smem<T>(h->tile_shape_dense, h->tile_warps_dense);
+    const size_t sm = force_smem<T>(S0, h->tile_warps), smd = force_smem<T>(S1, h->tile_warps_dense);
     int* cnt = h->defer + h->ntiles;
     cudaMemsetAsync(cnt, 0, sizeof(int), st);
 #define DPDE_FORCE(LMV)                                                                                           \
-    k_force_tile<T, LMV><<<g, blk, sm, st>>>(C, h->tile_org, h->tile_dim, half_dt, kick, h->tile_shape,           \
+    k_force_tile<T, LMV><<<g, blk, sm, st>>>(C, h->tile_org, h->tile_dim, half_dt, kick, S0,                      \
                                              h->frames, h->defer, cnt);                                           \
     k_force_tile_dense<T, LMV><<<gd, bd, smd, st>>> (C, h->tile_org, h->tile_dim, half_dt, kick,                  \
-                                                     h->tile_shape_dense, h->frames, h->defer, cnt)
+                                                     S1, h->frames, h->defer, cnt)
     switch (list) {
     case LIST_ALL: DPDE_FORCE(LIST_ALL); break;
     case LIST_CROSS: DPDE_FORCE(LIST_CROSS); break;
     case LIST_FWD: DPDE_FORCE(LIST_FWD); break;
+    case LIST_OBS: DPDE_FORCE(LIST_OBS); break;
     default: DPDE_FORCE(LIST_NONE); break;
     }
 #undef DPDE_FORCE
@@ -499,6 +508,7 @@ void enqueue_get_state(dpde_handle* h, cudaStream_t st, double* q, double* p, do
 template <class T>
 void enqueue_obs(dpde_handle* h, cudaStream_t st) {
     const Ctx<T> C = make_ctx<T>(h);
+    if (h->N > 0) enqueue_force<T>(h, C, st, T(0), 0, LIST_OBS);
     if (h->nchunks > 0)
         k_obs_chunks<T><<<h->nchunks, OBS_THREADS, 0, st>>>(C, h->chunk_rep, h->chunk_begin, h->chunk_end,
                                                              h->partial);
@@ -606,7 +616,7 @@ int set_tiles(dpde_handle* h, int edge) {
         if (!(big || few) || w[a] == 1) break;
         w[a] = (w[a] + 1) / 2;
     }
-    const size_t smem_limit = 200 * 1024;
+    const size_t smem_limit = FORCE_SMEM_MAX;
     // regular capacity 1.08x the mean halo + 64 (over 4 standard deviations
     // of a uniform fluid's count), deferred tiles 2.5x the mean
     auto capped = [&](double halo) {
@@ -664,6 +674,8 @@ int set_tiles(dpde_handle* h, int edge) {
         CK(h, cudaFuncSetAttribute(k_force_tile_dense<float, LIST_ALL>, A, smd));
         CK(h, cudaFuncSetAttribute(k_force_tile_dense<float, LIST_CROSS>, A, smd));
         CK(h, cudaFuncSetAttribute(k_force_tile_dense<float, LIST_FWD>, A, smd));
+        CK(h, cudaFuncSetAttribute(k_force_tile<float, LIST_OBS>, A, (int)FORCE_SMEM_MAX));
+        CK(h, cudaFuncSetAttribute(k_force_tile_dense<float, LIST_OBS>, A, (int)FORCE_SMEM_MAX));
     } else {
         CK(h, cudaFuncSetAttribute(k_force_tile<double, LIST_NONE>, A, sm));
         CK(h, cudaFuncSetAttribute(k_force_tile<double, LIST_ALL>, A, sm));
@@ -673,6 +685,8 @@ int set_tiles(dpde_handle* h, int edge) {
         CK(h, cudaFuncSetAttribute(k_force_tile_dense<double, LIST_ALL>, A, smd));
         CK(h, cudaFuncSetAttribute(k_force_tile_dense<double, LIST_CROSS>, A, smd));
         CK(h, cudaFuncSetAttribute(k_force_tile_dense<double, LIST_FWD>, A, smd));
+        CK(h, cudaFuncSetAttribute(k_force_tile<double, LIST_OBS>, A, (int)FORCE_SMEM_MAX));
+        CK(h, cudaFuncSetAttribute(k_force_tile_dense<double, LIST_OBS>, A, (int)FORCE_SMEM_MAX));
     }
     h->ntiles = (int)torg.size();
     h->frames = FrameTiles{h->frame_org, h->frame_rel, (int)forg.size(), edge, hframe};
@@ -1029,6 +1043,8 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
         CKC(cudaMemset(h->pA, 0, vsz * n1));
         CKC(cudaMemset(h->cA, 0, sizeof(int) * n1));
         CKC(cudaMemset(h->F, 0, vsz * n1));
+        CKC(cudaMemset(h->dp, 0, vsz * n1));
+        CKC(cudaMemset(h->start, 0, sizeof(int) * (c1 + 1)));
         CKC(cudaMemset(h->nbr_n, 0, sizeof(int) * n1));
         CKC(cudaMemset(h->fwd_n, 0, sizeof(int) * n1));
     }

