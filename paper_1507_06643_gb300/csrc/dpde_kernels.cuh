@@ -462,7 +462,21 @@ __global__ void k_copy_back(Ctx<T> C) {
 // pass however uneven the lists are. The pair values of one owner are summed
 // by a segmented shuffle scan (in entry order inside a pass, passes in order:
 // deterministic) and handed to the owner lane.
+//
+// What bounds them: the load/store unit, then issue. The lists are
+// entry-major, one row of a warp's particles contiguous, but a pass takes
+// several entries of one owner, so reading entries (and writing delta p_ij)
+// at [k N + i] touched a sector per lane, ~130 wavefronts a pass. The first
+// sweep now reads its lists a lane per owner, rows contiguous, into shared
+// memory in flat order (SERWIN_BYTES a warp: the ~400 entries of a warp at
+// density 3 in one window), and writes delta p_ij in flat order too, the
+// partner and the owner lane in the fourth word, so that the second sweep
+// reads one contiguous row a pass and no list. Us per step, first and second
+// sweep: SER at 1M 168 + 160 -> 144 + 88, Hybrid at 4M 193 + 196 -> 169 + 133.
 // ---------------------------------------------------------------------------
+constexpr int SER_THREADS = 128;
+constexpr int SERWIN_BYTES = 4096;
+
 struct WarpEntries {
     int lane, nn, incl, total;
 };
@@ -482,28 +496,31 @@ __device__ __forceinline__ WarpEntries warp_entries(int nn) {
     return W;
 }
 
-// owner lane of flat entry f (the first lane whose inclusive prefix exceeds f)
-// and the entry's index k in the owner's list
-__device__ __forceinline__ void warp_entry_owner(const WarpEntries& W, int f, int& owner, int& k) {
-    int lo = 0;
-#pragma unroll
-    for (int st = 16; st > 0; st >>= 1) {
-        const int v = __shfl_sync(0xffffffffu, W.incl, lo + st - 1);
-        if (v <= f) lo += st;
-    }
-    owner = lo;
-    k = f - __shfl_sync(0xffffffffu, W.incl - W.nn, lo);
+// partner slot and owner lane in one word
+static_assert(NBR_J_BITS == 27, "five bits hold the owner lane");
+__device__ __forceinline__ uint32_t pack_owner(int j, int lane) { return (uint32_t)j | ((uint32_t)lane << NBR_J_BITS); }
+__device__ __forceinline__ int owner_of(uint32_t x) { return (int)(x >> NBR_J_BITS); }
+__device__ __forceinline__ int partner_of(uint32_t x) { return (int)(x & ((1u << NBR_J_BITS) - 1)); }
+__device__ __forceinline__ uint32_t word_bits(float w) { return __float_as_uint(w); }
+__device__ __forceinline__ uint32_t word_bits(double w) { return (uint32_t)__double_as_longlong(w); }
+__device__ __forceinline__ void set_word(float& w, uint32_t x) { w = __uint_as_float(x); }
+__device__ __forceinline__ void set_word(double& w, uint32_t x) { w = __longlong_as_double((long long)x); }
+
+// first lane of my lane's run of equal owners
+__device__ __forceinline__ int owner_head(int lane, int owner) {
+    const int prev = __shfl_up_sync(0xffffffffu, owner, 1);
+    const uint32_t heads = __ballot_sync(0xffffffffu, lane == 0 || prev != owner);
+    return 31 - __clz((int)(heads & (0xffffffffu >> (31 - lane))));
 }
 
 // segmented sum of v over lanes with equal owner; returns to every lane the
 // sum over this pass's entries of its own particle (0 if none)
 template <class T>
-__device__ __forceinline__ T warp_owner_sum(const WarpEntries& W, int f0, int owner, T v) {
+__device__ __forceinline__ T warp_owner_sum(const WarpEntries& W, int f0, int head, T v) {
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const T y = __shfl_up_sync(0xffffffffu, v, o);
-        const int oy = __shfl_up_sync(0xffffffffu, owner, o);
-        if (W.lane >= o && oy == owner) v += y;
+        if (W.lane - o >= head) v += y;
     }
     // my entries in this pass end at flat index incl - 1
     const int last = W.incl - 1 - f0;
@@ -512,13 +529,10 @@ __device__ __forceinline__ T warp_owner_sum(const WarpEntries& W, int f0, int ow
     return mine ? s : T(0);
 }
 
-// delta p_ij of list entry k of particle i (pair arithmetic of Eq. SER_p)
+// delta p_ij of entry (j, w) of particle i (pair arithmetic of Eq. SER_p)
 template <class T>
-__device__ __forceinline__ T3<T> ser_dp(const Ctx<T>& C, int i, int k, uint32_t step, T dt, T sdt,
+__device__ __forceinline__ T3<T> ser_dp(const Ctx<T>& C, int j, T w, uint32_t step, T dt, T sdt,
                                         const vec_t<T>& pi, uint32_t idi, int rep) {
-    const ListEnt<T> en = C.nbr[(size_t)k * C.N + i];
-    const int j = en.j;
-    const T w = en.w;
     const vec_t<T> pj = C.pB[j];
     const T3<T> G = pair_gauss<T>(C.seed, step, (uint32_t)rep, idi, C.idB[j]);
     const T A = -(C.sig2_4 * (pi.w + pj.w)) * (w * w) * dt;
@@ -528,35 +542,62 @@ __device__ __forceinline__ T3<T> ser_dp(const Ctx<T>& C, int i, int k, uint32_t 
 }
 
 // first sweep: delta p_i = sum_j delta p_ij (Eq. SER_p). Each delta p_ij is
-// also written, entry-major like the list, into the forward-entry buffer
-// fwd_g (free once the SSA part of the step is done), so that the second
+// also written, with its partner and owner, into the forward-entry buffer
+// fwd_g (free once the SSA part of the step is done), the entries of a warp's
+// particles in flat order from [first particle * cap], so that the second
 // sweep reads it instead of drawing the pair's Gaussian again.
 template <class T>
-__global__ void k_ser_sweep1(Ctx<T> C, T dt, T sqrt_dt) {
+__global__ void __launch_bounds__(SER_THREADS) k_ser_sweep1(Ctx<T> C, T dt, T sqrt_dt) {
+    constexpr int WIN = SERWIN_BYTES / (int)sizeof(ListEnt<T>);   // entries held at a time (a multiple of 32)
+    __shared__ ListEnt<T> win[SER_THREADS / 32][WIN];
+    ListEnt<T>* const ent = win[threadIdx.x >> 5];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int base = i - (int)(threadIdx.x & 31);
     const WarpEntries W = warp_entries(i < C.N ? C.nbr_n[i] : 0);
     const uint32_t step = (uint32_t)*C.step;
     const T sdt = C.sigma * sqrt_dt;
+    const size_t N = (size_t)C.N;
+    const int excl = W.incl - W.nn;
+    vec_t<T>* const out_g = C.fwd_g + (size_t)base * C.nbr_cap;
     T ax = 0, ay = 0, az = 0;
-    for (int f0 = 0; f0 < W.total; f0 += 32) {
-        const int f = f0 + W.lane;
-        int o, k;
-        warp_entry_owner(W, f, o, k);
-        T3<T> d{0, 0, 0};
-        if (f < W.total) {
-            const int io = base + o;
-            d = ser_dp(C, io, k, step, dt, sdt, C.pB[io], C.idB[io], C.rep_of_slot[io]);
-            // kept for the second sweep, entry-major like the list
-            vec_t<T> dv;
-            dv.x = d.x; dv.y = d.y; dv.z = d.z; dv.w = T(0);
-            C.fwd_g[(size_t)k * C.N + io] = dv;
-        } else {
-            o = 32;
+    for (int c0 = 0; c0 < W.total; c0 += WIN) {
+        // my entries of the window, four loads in flight (past the end the
+        // last one again)
+        const int k1 = min(W.nn, c0 + WIN - excl);
+        const ListEnt<T>* row = C.nbr + i;
+        for (int k = max(0, c0 - excl); k < k1; k += 4) {
+            ListEnt<T> v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = row[(size_t)min(k + u, k1 - 1) * N];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k + u < k1) {
+                    v[u].j = (int)pack_owner(v[u].j, W.lane);
+                    ent[excl + k + u - c0] = v[u];
+                }
         }
-        ax += warp_owner_sum(W, f0, o, d.x);
-        ay += warp_owner_sum(W, f0, o, d.y);
-        az += warp_owner_sum(W, f0, o, d.z);
+        __syncwarp();
+        const int end = min(W.total, c0 + WIN);
+        for (int f0 = c0; f0 < end; f0 += 32) {
+            const int f = f0 + W.lane;
+            int o = 32;
+            T3<T> d{0, 0, 0};
+            if (f < end) {
+                const ListEnt<T> en = ent[f - c0];
+                o = owner_of((uint32_t)en.j);
+                const int io = base + o;
+                d = ser_dp(C, partner_of((uint32_t)en.j), en.w, step, dt, sdt, C.pB[io], C.idB[io], C.rep_of_slot[io]);
+                vec_t<T> dv;
+                dv.x = d.x; dv.y = d.y; dv.z = d.z;
+                set_word(dv.w, (uint32_t)en.j);
+                out_g[f] = dv;
+            }
+            const int head = owner_head(W.lane, o);
+            ax += warp_owner_sum(W, f0, head, d.x);
+            ay += warp_owner_sum(W, f0, head, d.y);
+            az += warp_owner_sum(W, f0, head, d.z);
+        }
+        __syncwarp();   // the window has been read
     }
     if (i >= C.N) return;
     vec_t<T> out;
@@ -602,35 +643,33 @@ __device__ __forceinline__ ff eps_minus_dk(ff e, ff add, const float4& pn, const
 // conserves energy up to the rounding of per-particle sums. Writes the new
 // state (q, cell, p, eps) into set A.
 template <class T>
-__global__ void k_ser_sweep2(Ctx<T> C, T dt, T sqrt_dt) {
+__global__ void __launch_bounds__(SER_THREADS) k_ser_sweep2(Ctx<T> C) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int base = i - (int)(threadIdx.x & 31);
     const WarpEntries W = warp_entries(i < C.N ? C.nbr_n[i] : 0);
-    const uint32_t step = (uint32_t)*C.step;
-    const T sdt = C.sigma * sqrt_dt;
     const T hm = T(0.5) * C.inv_m;
+    const vec_t<T>* const in_g = C.fwd_g + (size_t)base * C.nbr_cap;   // delta p_ij of the first sweep
     eps_t<T> tsum{};   // compensated in the mixed mode
     for (int f0 = 0; f0 < W.total; f0 += 32) {
         const int f = f0 + W.lane;
-        int o, k;
-        warp_entry_owner(W, f, o, k);
+        int o = 32;
         T tv = 0;
         if (f < W.total) {
-            const int io = base + o;
+            const vec_t<T> d = in_g[f];
+            const uint32_t jo = word_bits(d.w);
+            o = owner_of(jo);
+            const int io = base + o, j = partner_of(jo);
             const vec_t<T> pi = C.pB[io];
             const vec_t<T> dpi = C.dp[io];
-            const int j = C.nbr[(size_t)k * C.N + io].j;
-            const vec_t<T> d = C.fwd_g[(size_t)k * C.N + io];   // delta p_ij of the first sweep
             const vec_t<T> pj = C.pB[j];
             const vec_t<T> dpj = C.dp[j];
             const T vix = pi.x * C.inv_m, viy = pi.y * C.inv_m, viz = pi.z * C.inv_m;
             const T vjx = pj.x * C.inv_m, vjy = pj.y * C.inv_m, vjz = pj.z * C.inv_m;
             tv = d.x * ((vix + vjx) + (dpi.x + dpj.x) * hm) + d.y * ((viy + vjy) + (dpi.y + dpj.y) * hm) +
                  d.z * ((viz + vjz) + (dpi.z + dpj.z) * hm);
-        } else {
-            o = 32;
         }
-        tsum = eps_add(tsum, warp_owner_sum(W, f0, o, tv));
+        const int head = owner_head(W.lane, o);
+        tsum = eps_add(tsum, warp_owner_sum(W, f0, head, tv));
     }
     if (i >= C.N) return;
     const RepInfo& R = C.reps[C.rep_of_slot[i]];
