@@ -132,6 +132,7 @@ struct dpde_handle {
     RepInfo* d_reps = nullptr;
     long long* d_step = nullptr;
     unsigned int* d_status = nullptr;
+    double2* gauss_tab = nullptr;    // tables of the Gaussians (FP64)
     double* staging = nullptr;       // 7N doubles: q (3N), p (3N), eps (N)
     int* cells_out = nullptr;        // 3N ints (diagnostic)
     long long step = 0;              // host mirror of the device counter
@@ -186,7 +187,7 @@ Ctx<T> make_ctx(dpde_handle* h) {
     C.a = (T)h->prm.a; C.sigma = (T)h->prm.sigma;
     C.pot = cast_pot<T>(make_pot(h->prm.potential, h->prm.a, h->prm.r_cut, h->prm.lj_eps, h->prm.lj_r));
     C.sig2_4 = (T)(h->prm.sigma * h->prm.sigma / 4.0);
-    C.seed = philox_keys(make_uint2((uint32_t)(h->prm.seed & 0xffffffffu), (uint32_t)(h->prm.seed >> 32)));
+    C.seed = philox_keys(make_uint2((uint32_t)(h->prm.seed & 0xffffffffu), (uint32_t)(h->prm.seed >> 32)), h->gauss_tab);
     return C;
 }
 
@@ -541,7 +542,7 @@ void free_all(dpde_handle* h) {
                     h->nbr_n, h->fwd_g, h->fwd_n, h->tile_org, h->tile_dim, h->frame_org, h->frame_rel, h->defer, h->col_cells[0], h->col_cells[1], h->dom_cells, h->dom_off, h->dom_cell0, h->rdom_cells, h->rdom_off, h->rdom_cell0, h->lv_off, h->lv_n, h->ssa_defer, h->d_col_off[0], h->d_col_off[1], h->d_bar, h->wallpos, h->idB, h->key, h->tmp, h->cnt, h->start, h->bsum, h->rep_of_slot,
                     h->rep_of_cell, h->brick_rep, h->tab, h->chunk_rep, h->chunk_begin, h->chunk_end,
                     h->rep_chunk_begin, h->partial, h->obs_out, h->d_reps, h->d_step, h->d_status,
-                    h->staging, h->cells_out};
+                    h->staging, h->cells_out, h->gauss_tab};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
@@ -1015,6 +1016,11 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
     CKC(cudaMalloc(&h->wallpos, sizeof(WallPos) * (size_t)std::max(1, h->R)));
     CKC(cudaMalloc(&h->d_step, sizeof(long long)));
     CKC(cudaMalloc(&h->d_status, sizeof(unsigned int)));
+    if (!h->mixed) {
+        const std::vector<double2>& t = gauss_tables();
+        CKC(cudaMalloc(&h->gauss_tab, sizeof(double2) * t.size()));
+        CKC(cudaMemcpy(h->gauss_tab, t.data(), sizeof(double2) * t.size(), cudaMemcpyHostToDevice));
+    }
     CKC(cudaMalloc(&h->staging, sizeof(double) * 7 * n1));
     CKC(cudaMalloc(&h->cells_out, sizeof(int) * 3 * n1));
     {
@@ -1582,21 +1588,25 @@ int dpde_debug_gaussian(int64_t n, uint64_t seed, const uint32_t* step, const ui
     if (n == 0) return DPDE_OK;
     uint32_t* d = nullptr;
     double* dout = nullptr;
+    double2* dtab = nullptr;
+    const std::vector<double2>& tab = gauss_tables();
     cudaError_t e = cudaMalloc(&d, 16 * (size_t)n);
     if (e == cudaSuccess) e = cudaMalloc(&dout, 24 * (size_t)n);
+    if (e == cudaSuccess) e = cudaMalloc(&dtab, sizeof(double2) * tab.size());
+    if (e == cudaSuccess) e = cudaMemcpy(dtab, tab.data(), sizeof(double2) * tab.size(), cudaMemcpyHostToDevice);
     const uint32_t* src[4] = {step, replica, id_a, id_b};
     for (int k = 0; k < 4 && e == cudaSuccess; ++k)
         e = cudaMemcpy(d + (size_t)k * n, src[k], 4 * (size_t)n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
         const uint2 s = make_uint2((uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32));
         if (precision == DPDE_FP64)
-            k_debug_gauss<double><<<ceil_div(n, 256), 256>>>((int)n, s, d, d + n, d + 2 * n, d + 3 * n, dout);
+            k_debug_gauss<double><<<ceil_div(n, 256), 256>>>((int)n, s, dtab, d, d + n, d + 2 * n, d + 3 * n, dout);
         else
-            k_debug_gauss<float><<<ceil_div(n, 256), 256>>>((int)n, s, d, d + n, d + 2 * n, d + 3 * n, dout);
+            k_debug_gauss<float><<<ceil_div(n, 256), 256>>>((int)n, s, dtab, d, d + n, d + 2 * n, d + 3 * n, dout);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpy(out, dout, 24 * (size_t)n, cudaMemcpyDeviceToHost);
-    cudaFree(d); cudaFree(dout);
+    cudaFree(d); cudaFree(dout); cudaFree(dtab);
     if (e != cudaSuccess) return fail(nullptr, DPDE_ERR_CUDA, cudaGetErrorString(e));
     return DPDE_OK;
 }

@@ -20,6 +20,7 @@
 #include <cmath>
 
 #include <cstdint>
+#include <vector>
 #include <cuda_runtime.h>
 
 namespace dpde {
@@ -155,12 +156,15 @@ template <> __device__ __forceinline__ float cell_len<float>(const RepInfo& R, i
 //
 // The ten round keys of a handle's seed are launch constants (kernel
 // parameters): bumping the key in every draw was 18 of its ~300 instructions.
+// tab: the tables of the double-precision Gaussians (gauss_tables).
 struct PhiloxKeys {
     uint32_t x[10], y[10];
+    const double2* tab;
 };
 
-__host__ __device__ __forceinline__ PhiloxKeys philox_keys(uint2 k) {
+__host__ __device__ __forceinline__ PhiloxKeys philox_keys(uint2 k, const double2* tab = nullptr) {
     PhiloxKeys K;
+    K.tab = tab;
     for (int r = 0; r < 10; ++r) {
         K.x[r] = k.x + (uint32_t)r * 0x9E3779B9u;
         K.y[r] = k.y + (uint32_t)r * 0xBB67AE85u;
@@ -184,7 +188,7 @@ template <class T> struct T3 { T x, y, z; };
 
 // Box-Muller on 24-bit uniforms u in (0, 1] and t in [0, 1) (exact in float):
 // G = (R1 cos 2 pi t1, R1 sin 2 pi t1, R2 cos 2 pi t2), R = sqrt(-2 ln u).
-__device__ __forceinline__ T3<float> gauss3(uint4 x, float) {
+__device__ __forceinline__ T3<float> gauss3(uint4 x, const double2*, float) {
     const float u1 = (float)((x.x >> 8) + 1u) * 0x1p-24f;
     const float t1 = (float)(x.y >> 8) * 0x1p-24f;
     const float u2 = (float)((x.z >> 8) + 1u) * 0x1p-24f;
@@ -196,17 +200,91 @@ __device__ __forceinline__ T3<float> gauss3(uint4 x, float) {
     const float c2 = cospif(2.0f * t2);
     return {R1 * c1, R1 * s1, R2 * c2};
 }
-__device__ __forceinline__ T3<double> gauss3(uint4 x, double) {
-    const double u1 = (double)((x.x >> 8) + 1u) * 0x1p-24;
-    const double t1 = (double)(x.y >> 8) * 0x1p-24;
-    const double u2 = (double)((x.z >> 8) + 1u) * 0x1p-24;
-    const double t2 = (double)(x.w >> 8) * 0x1p-24;
-    const double R1 = sqrt(-2.0 * log(u1));
-    const double R2 = sqrt(-2.0 * log(u2));
-    double s1, c1;
-    sincospi(2.0 * t1, &s1, &c1);
-    const double c2 = cospi(2.0 * t2);
-    return {R1 * c1, R1 * s1, R2 * c2};
+
+// In double the chip does two operations a clock and SM, so their count is the
+// time (log, sincospi and cospi were ~120 of a draw's): both functions are
+// table-driven (P. T. P. Tang, ACM TOMS 15 (1989) and 16 (1990)), which the
+// 24-bit arguments suit.
+//   -2 ln(K / 2^24): K = 2^e m, m in [1, 2) in 512 intervals with reciprocals
+//     c of 26 bits, so that r = m c - 1, |r| < 2^-9, is exact; the sum of
+//     -2 E ln 2 and -2 L (L = -ln c, less ln 2 from sqrt(2) on, where E counts
+//     one more) is exact in the tables' high parts, multiples of 2^-42.
+//   angle 2 pi T / 2^24: folded to an eighth of a turn, 512 steps, and the
+//     Taylor series of sine and cosine for the rest, at most 7.7e-4.
+// Errors of ln, cos and sin: 1 to 2 ulp, as CUDA's. Us per pass in FP64: ten
+// Hybrid steps of 1,000 particles 5445 -> 5024, two of 108,000 2183 -> 2030.
+constexpr int GT_TRIG = 0, GT_TRIG_N = 513;             // (cos, sin)
+constexpr int GT_EXP = GT_TRIG + GT_TRIG_N, GT_EXP_N = 25;   // (high, low) of 2 (24 - E) ln 2, E = 0..24
+constexpr int GT_LOG = GT_EXP + GT_EXP_N, GT_LOG_N = 512;    // (c, high), (low, 0)
+constexpr int GT_SIZE = GT_LOG + 2 * GT_LOG_N;
+constexpr int GT_FOLD = 212;                             // first interval beyond sqrt(2)
+
+// the tables, built on the host once (0.7 ms where long double is software)
+inline std::vector<double2> make_gauss_tables() {
+    std::vector<double2> t(GT_SIZE);
+    const long double pi = 3.14159265358979323846264338327950288L, ln2 = std::log(2.0L);
+    auto split = [](long double x) {
+        const double hi = (double)(std::nearbyint(x * 0x1p42L) * 0x1p-42L);
+        return make_double2(hi, (double)(x - (long double)hi));
+    };
+    for (int i = 0; i < GT_TRIG_N; ++i)
+        t[GT_TRIG + i] = make_double2((double)std::cos(pi * i / 2048), (double)std::sin(pi * i / 2048));
+    for (int e = 0; e < GT_EXP_N; ++e) t[GT_EXP + e] = split(2 * (24 - e) * ln2);
+    for (int i = 0; i < GT_LOG_N; ++i) {
+        // c = 1 and 1/2 at the ends, so that ln 1 = 0 is met without cancellation
+        const double c = i == 0 ? 1.0 : (i == GT_LOG_N - 1 ? 0.5 : std::nearbyint(0x1p26 / (1.0 + (i + 0.5) / 512)) * 0x1p-26);
+        const double2 l = split(2 * std::log((long double)c * (i < GT_FOLD ? 1 : 2)));
+        t[GT_LOG + 2 * i] = make_double2(c, l.x);
+        t[GT_LOG + 2 * i + 1] = make_double2(l.y, 0.0);
+    }
+    return t;
+}
+inline const std::vector<double2>& gauss_tables() {
+    static const std::vector<double2> t = make_gauss_tables();
+    return t;
+}
+
+__device__ __forceinline__ double neg2_log24(uint32_t K, const double2* __restrict__ tab) {   // 1 <= K <= 2^24
+    const uint32_t f = __float_as_uint((float)K);   // exact
+    const uint32_t mant = f & 0x7fffffu, i = mant >> 14;
+    const int E = (int)(f >> 23) - 127 + (i >= (uint32_t)GT_FOLD ? 1 : 0);
+    const double m = __hiloint2double((int)(0x3ff00000u | (mant >> 3)), (int)(mant << 29));
+    const double2 a = tab[GT_LOG + 2 * i], x = tab[GT_EXP + E];
+    const double lo = tab[GT_LOG + 2 * i + 1].x + x.y;
+    const double r = fma(m, a.x, -1.0);
+    double q = fma(r, 2.0 / 6, -2.0 / 5);   // -2 log1p(r) / r
+    q = fma(r, q, 2.0 / 4);
+    q = fma(r, q, -2.0 / 3);
+    q = fma(r, q, 1.0);
+    q = fma(r, q, -2.0);
+    return (x.x + a.y) + fma(r, q, lo);
+}
+
+// cos and sin of 2 pi T / 2^24, T < 2^24
+__device__ __forceinline__ double2 cos_sin24(uint32_t T, const double2* __restrict__ tab) {
+    const uint32_t quad = T >> 22;
+    uint32_t f = T & 0x3fffffu;
+    const bool fold = f > 0x200000u;   // beyond 45 degrees: the complement
+    f = fold ? 0x400000u - f : f;
+    const uint32_t i = (f + 2048u) >> 12;
+    const double2 a = tab[GT_TRIG + i];
+    // times 2 pi / 2^24 in two parts, the first of 40 bits: an exact product
+    const double n = (double)((int)f - (int)(i << 12)), b = fma(n, 0x1.a308d313198a3p-63, n * 0x1.921fb54442000p-22);
+    const double b2 = b * b;
+    const double sb = fma(b * b2, fma(b2, 1.0 / 120, -1.0 / 6), b);
+    const double cb = b2 * fma(b2, 1.0 / 24, -0.5);   // cos b - 1
+    double c = fma(-a.y, sb, fma(a.x, cb, a.x));
+    double s = fma(a.x, sb, fma(a.y, cb, a.y));
+    const bool swap = fold != ((quad & 1) != 0);   // odd quadrants: (cos, sin) -> (-sin, cos)
+    const double c1 = swap ? s : c, s1 = swap ? c : s;
+    return make_double2(quad == 1 || quad == 2 ? -c1 : c1, quad >= 2 ? -s1 : s1);
+}
+
+__device__ __forceinline__ T3<double> gauss3(uint4 x, const double2* __restrict__ tab, double) {
+    const double R1 = sqrt(neg2_log24((x.x >> 8) + 1u, tab));
+    const double R2 = sqrt(neg2_log24((x.z >> 8) + 1u, tab));
+    const double2 t1 = cos_sin24(x.y >> 8, tab);
+    return {R1 * t1.x, R1 * t1.y, R2 * cos_sin24(x.w >> 8, tab).x};
 }
 
 // G_ij for particle i (id_i) and neighbour j (id_j): drawn for the ordered
@@ -216,7 +294,7 @@ __device__ __forceinline__ T3<T> pair_gauss(const PhiloxKeys& key, uint32_t step
                                             uint32_t id_j) {
     const bool lo = id_i < id_j;
     const uint4 x = philox4x32_10(make_uint4(lo ? id_i : id_j, lo ? id_j : id_i, step, rep), key);
-    T3<T> g = gauss3(x, T(0));
+    T3<T> g = gauss3(x, key.tab, T(0));
     if (!lo) {
         g.x = -g.x;
         g.y = -g.y;

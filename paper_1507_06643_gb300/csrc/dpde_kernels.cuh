@@ -1372,12 +1372,12 @@ __global__ void k_debug_philox(int n, const uint4* __restrict__ ctr, const uint2
 }
 
 template <class T>
-__global__ void k_debug_gauss(int n, uint2 seed, const uint32_t* __restrict__ step,
+__global__ void k_debug_gauss(int n, uint2 seed, const double2* tab, const uint32_t* __restrict__ step,
                               const uint32_t* __restrict__ rep, const uint32_t* __restrict__ a,
                               const uint32_t* __restrict__ b, double* __restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const T3<T> g = pair_gauss<T>(philox_keys(seed), step[i], rep[i], a[i], b[i]);
+    const T3<T> g = pair_gauss<T>(philox_keys(seed, tab), step[i], rep[i], a[i], b[i]);
     out[3 * i] = g.x; out[3 * i + 1] = g.y; out[3 * i + 2] = g.z;
 }
 
