@@ -60,9 +60,6 @@ template <class T> struct Ctx {
 // ---------------------------------------------------------------------------
 // small helpers
 // ---------------------------------------------------------------------------
-template <class T> __device__ __forceinline__ T texpm1(T x);
-template <> __device__ __forceinline__ float texpm1(float x) { return expm1f(x); }
-template <> __device__ __forceinline__ double texpm1(double x) { return expm1(x); }
 template <class T> __device__ __forceinline__ T tfloor(T x);
 template <> __device__ __forceinline__ float tfloor(float x) { return floorf(x); }
 template <> __device__ __forceinline__ double tfloor(double x) { return floor(x); }
@@ -809,12 +806,11 @@ __global__ void k_ssa_gauss(Ctx<T> C) {
 // beta = C_v / eps: exact in double; in float through the fast reciprocal
 // (2 ulp), which keeps the chains' critical path short
 __device__ __forceinline__ float ssa_beta(ff e, const RepInfo& R) { return __fdividef(R.cvf, e.hi); }
-// sqrt(x / y) for x >= 0, y > 0: exact in double; in float x rsqrt(x y) (a
-// few ulp, for x y a normal float; 0 for x = 0)
+// sqrt(x / y) for x >= 0, y > 0 as x rsqrt(x y) (a few ulp, for x y a normal
+// float; 0 for x = 0)
 __device__ __forceinline__ float ssa_sqrt_ratio(float x, float y) {
     return x > 0.0f ? __fmul_rn(x, rsqrtf(__fmul_rn(x, y))) : 0.0f;
 }
-__device__ __forceinline__ double ssa_sqrt_ratio(double x, double y) { return sqrt(x / y); }
 __device__ __forceinline__ double ssa_beta(double e, const RepInfo& R) { return R.cv / e; }
 
 // Explicitly rounded operations: the compiler neither fuses nor reorders them,
@@ -828,22 +824,83 @@ __device__ __forceinline__ double r_mul(double a, double b) { return __dmul_rn(a
 __device__ __forceinline__ float r_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double r_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// k2 = 2 dt / m
+// In double an operation takes the chip some thirty times a float's, so a
+// map's count of them is its time. With a = gamma w^2 2 dt / m the amplitude
+// sigma sqrt(m (1 - e^{-2a}) / gamma) is 2 sigma sqrt(dt) w Q(a),
+//   Q(a) = sqrt((1 - e^{-2a}) / (2a)),
+// which needs neither the division nor the root where a is small: there
+// (e^{-a} - 1) / 2 and Q are polynomials (Chebyshev fits on [0, 1/4], error
+// below 2^-56), independent of each other. What does not depend on the state
+// goes into the map's noise (ssa_noise) beforehand. a is 0.02 to 0.2 in the
+// fluids of the paper; beyond 1/4 the functions themselves. Us per pass: ten
+// Hybrid steps of 1,000 particles 5024 -> 3936, two of 108,000 2030 -> 1802.
+__device__ __forceinline__ void ssa_ou(double a, double& hem, double& Q) {
+    if (a >= 0.0 && a <= 0.25) {
+        double h = 1.23028890849153e-07;
+        h = fma(a, h, -1.3701804316291336e-06);
+        h = fma(a, h, 1.2398555234119672e-05);
+        h = fma(a, h, -9.920595362410088e-05);
+        h = fma(a, h, 0.000694444401087605);
+        h = fma(a, h, -0.0041666666637702535);
+        h = fma(a, h, 0.02083333333322211);
+        h = fma(a, h, -0.08333333333333116);
+        h = fma(a, h, 0.24999999999999997);
+        h = fma(a, h, -0.5);
+        hem = __dmul_rn(a, h);
+        double q = 6.5425756532649734e-06;
+        q = fma(a, q, -5.837075404796853e-05);
+        q = fma(a, q, 0.0003668523284567146);
+        q = fma(a, q, -0.002343749303760139);
+        q = fma(a, q, 0.013715277715415457);
+        q = fma(a, q, -0.06249999999689911);
+        q = fma(a, q, 0.20833333333325674);
+        q = fma(a, q, -0.4999999999999993);
+        Q = fma(a, q, 1.0);
+    } else {
+        const double em1 = expm1(-a);
+        hem = __dmul_rn(0.5, em1);
+        Q = sqrt(__dmul_rn(em1, __dadd_rn(em1, 2.0)) / __dmul_rn(-2.0, a));
+    }
+}
+
+// The noise of a map from its entry (G, w), k2 = 2 dt / m, amp0 = 2 sigma
+// sqrt(dt): in double (amp0 w G / 2, sigma^2 / 4 w^2 k2), in float the entry.
+__device__ __forceinline__ float4 ssa_noise(const Ctx<float>&, const float4& g, float, float) { return g; }
+__device__ __forceinline__ d4 ssa_noise(const Ctx<double>& C, const d4& g, double k2, double amp0) {
+    const double A = __dmul_rn(0.5, __dmul_rn(amp0, g.w));
+    d4 n;
+    n.x = __dmul_rn(A, g.x);
+    n.y = __dmul_rn(A, g.y);
+    n.z = __dmul_rn(A, g.z);
+    n.w = __dmul_rn(C.sig2_4, __dmul_rn(__dmul_rn(g.w, g.w), k2));
+    return n;
+}
+
+// The map with its noise g.
 template <class T>
-__device__ __forceinline__ void ssa_pair_map(const Ctx<T>& C, const RepInfo& R, vec_t<T>& ps, eps_t<T>& es,
-                                             T& bs, vec_t<T>& pt, eps_t<T>& et, const vec_t<T>& g, T k2,
-                                             T amp0) {
-    const T w = g.w;
-    const T chik = r_mul(r_mul(w, w), k2);
-    const T gam = r_mul(C.sig2_4, r_add(bs, pt.w));
-    const T aa = r_mul(gam, chik);   // a = 2 gamma chi dt / m
-    // e^{-a} - 1, and 1 - e^{-2a} = -(e^{-a} - 1)(e^{-a} - 1 + 2)
-    const T em1 = texpm1(-aa);
-    const T x = r_mul(C.m, -r_mul(em1, r_add(em1, T(2))));   // m (1 - e^{-2a})
-    const T amp = (gam != T(0)) ? r_mul(C.sigma, ssa_sqrt_ratio(x, gam)) : r_mul(amp0, w);
-    const T Dx = r_mul(T(0.5), r_fma(em1, r_sub(ps.x, pt.x), r_mul(amp, g.x)));
-    const T Dy = r_mul(T(0.5), r_fma(em1, r_sub(ps.y, pt.y), r_mul(amp, g.y)));
-    const T Dz = r_mul(T(0.5), r_fma(em1, r_sub(ps.z, pt.z), r_mul(amp, g.z)));
+__device__ __forceinline__ void ssa_noise_map(const Ctx<T>& C, const RepInfo& R, vec_t<T>& ps, eps_t<T>& es,
+                                              T& bs, vec_t<T>& pt, eps_t<T>& et, const vec_t<T>& g, T k2,
+                                              T amp0) {
+    T Dx, Dy, Dz;
+    if constexpr (sizeof(T) == 8) {
+        T hem, Q;
+        ssa_ou(r_mul(g.w, r_add(bs, pt.w)), hem, Q);
+        Dx = r_fma(hem, r_sub(ps.x, pt.x), r_mul(Q, g.x));
+        Dy = r_fma(hem, r_sub(ps.y, pt.y), r_mul(Q, g.y));
+        Dz = r_fma(hem, r_sub(ps.z, pt.z), r_mul(Q, g.z));
+    } else {
+        const T w = g.w;
+        const T chik = r_mul(r_mul(w, w), k2);
+        const T gam = r_mul(C.sig2_4, r_add(bs, pt.w));
+        const T aa = r_mul(gam, chik);   // a = 2 gamma chi dt / m
+        // e^{-a} - 1, and 1 - e^{-2a} = -(e^{-a} - 1)(e^{-a} - 1 + 2)
+        const T em1 = expm1f(-aa);
+        const T x = r_mul(C.m, -r_mul(em1, r_add(em1, T(2))));   // m (1 - e^{-2a})
+        const T amp = (gam != T(0)) ? r_mul(C.sigma, ssa_sqrt_ratio((float)x, (float)gam)) : r_mul(amp0, w);
+        Dx = r_mul(T(0.5), r_fma(em1, r_sub(ps.x, pt.x), r_mul(amp, g.x)));
+        Dy = r_mul(T(0.5), r_fma(em1, r_sub(ps.y, pt.y), r_mul(amp, g.y)));
+        Dz = r_mul(T(0.5), r_fma(em1, r_sub(ps.z, pt.z), r_mul(amp, g.z)));
+    }
     const T snx = r_add(ps.x, Dx), sny = r_add(ps.y, Dy), snz = r_add(ps.z, Dz);
     const T tnx = r_sub(pt.x, Dx), tny = r_sub(pt.y, Dy), tnz = r_sub(pt.z, Dz);
     // kinetic-energy change of the stored momenta, halved
@@ -860,6 +917,14 @@ __device__ __forceinline__ void ssa_pair_map(const Ctx<T>& C, const RepInfo& R, 
     pt.x = tnx; pt.y = tny; pt.z = tnz;
     et = eps_add(et, -dK);
     pt.w = ssa_beta(et, R);
+}
+
+// The map of the entry (G, w) = g.
+template <class T>
+__device__ __forceinline__ void ssa_pair_map(const Ctx<T>& C, const RepInfo& R, vec_t<T>& ps, eps_t<T>& es,
+                                             T& bs, vec_t<T>& pt, eps_t<T>& et, const vec_t<T>& g, T k2,
+                                             T amp0) {
+    ssa_noise_map(C, R, ps, es, bs, pt, et, ssa_noise(C, g, k2, amp0), k2, amp0);
 }
 
 // Plain (unpipelined) chain, for cells with more than SSA_ROWS rows.

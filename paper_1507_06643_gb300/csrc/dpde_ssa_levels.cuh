@@ -355,6 +355,8 @@ __device__ __forceinline__ void ssa_exec_levels(const Ctx<T>& C, const SsaLevels
     const int E = lvs[nlev];
     const int nchunk = (E + SSA_CHUNK - 1) / SSA_CHUNK;
     const SsaRec<T>* rec = V.rec + (size_t)sb * C.nbr_cap;
+    const T amp0 = T(2) * C.sigma * sqrt_dt;   // amplitude of the map as gamma -> 0
+    const T k2 = T(2) * dt * C.inv_m;
     if (tid >= nmap) {
         // a record of every SSA_DRAW_THREADS, the next one loaded while this
         // one's Gaussian is drawn
@@ -372,15 +374,13 @@ __device__ __forceinline__ void ssa_exec_levels(const Ctx<T>& C, const SsaLevels
                 const T3<T> G = pair_gauss<T>(C.seed, step, (uint32_t)rep, ID[y.st & 0xffffu], ID[y.st >> 16]);
                 vec_t<T> g;
                 g.x = G.x; g.y = G.y; g.z = G.z; g.w = y.w;
-                ring[at] = g;
+                ring[at] = ssa_noise(C, g, k2, amp0);
                 ring_st[at] = y.st;
             }
             block_bar();
         }
         return;
     }
-    const T amp0 = T(2) * C.sigma * sqrt_dt;   // amplitude of the map as gamma -> 0
-    const T k2 = T(2) * dt * C.inv_m;
     // level ends: the current level's, and the next one's, read a step ahead
     int l = 1, lend = lvs[min(1, nlev)], lnext = lvs[min(2, nlev)];
     block_bar();                           // chunk 0 is drawn
@@ -428,7 +428,7 @@ __device__ __forceinline__ void ssa_exec_levels(const Ctx<T>& C, const SsaLevels
                 T bs = ps.w;
                 vec_t<T> pt = P[t];
                 eps_t<T> et = Es[t];
-                ssa_pair_map(C, R, ps, es, bs, pt, et, g, k2, amp0);
+                ssa_noise_map(C, R, ps, es, bs, pt, et, g, k2, amp0);
                 ps.w = bs;
                 P[s] = ps;
                 Es[s] = es;

@@ -1,10 +1,15 @@
-"""The double-precision draw (GPU) at the ends of its range.
+"""The double-precision draw and pair map (GPU) at the ends of their ranges.
 
 Gaussians: Box-Muller in long double on the uniforms of the oracle's Philox
 words, for many pairs; -2 ln u, cosine and sine are each within 4 ulp, so R c
-is within (4 / 2 + 4 + 1.5) ulp < 2e-15, relative to R."""
+is within (4 / 2 + 4 + 1.5) ulp < 2e-15, relative to R. Pair maps: two SSA
+steps against the oracle, where a = 2 gamma chi dt / m stays below 1/4 (the
+polynomials), spreads over both sides of it, and is large throughout, with
+the parity tests' 1e-11."""
 import numpy as np
 import pytest
+
+from gpu_util import assert_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -28,3 +33,9 @@ def test_gaussians_against_long_double():
     err = np.abs(got - ref) / np.stack([r1, r1, r2], 1)
     assert err.max() < 2e-15, err.max()
 
+
+@pytest.mark.parametrize("sigma,dt", [(3.0, 0.01), (5.0, 0.02), (10.0, 0.1), (0.0, 0.01)])
+def test_pair_map_ranges(sigma, dt):
+    specs = [(300, (4.7,) * 3, 50.0, 1.0, (1, 1, 1))]
+    for _ in assert_parity(specs, "fp64", "SSA", 2, 1e-11, (3, 4, 5), sigma=sigma, dt=dt, a=1.0):
+        pass
