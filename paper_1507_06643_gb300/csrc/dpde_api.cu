@@ -2,6 +2,7 @@
 // sequence of one timestep, CUDA-graph replay, observables, diagnostics.
 #include "dpde.h"
 #include "dpde_force.cuh"
+#include "dpde_ssa_cells.cuh"
 #include "dpde_ssa_levels.cuh"
 #include "dpde_ssa_persistent.cuh"
 
@@ -46,6 +47,11 @@ struct GraphKey {
 
 constexpr size_t FORCE_SMEM_MAX = 200 * 1024;   // dynamic shared memory of a force block, at most
 constexpr size_t SSA_ALONE_SMEM = 116 * 1024;   // one such block per SM
+// Cells of a colour class per SM up to which a warp takes a cell: its time is
+// that of the longest cell, ~10 us, until the warps fill the chip (SSA step at
+// density 3: 20,011 particles 442 -> 280 us, 64,000 642 -> 406, 200,000, 16
+// cells per SM, 898 -> 655; 1,000,000, 81 per SM, 1177 against 1764).
+constexpr int CELLS_SM = 32;
 constexpr int STATE_CHUNKS = 4;   // chunks of a host <-> device state transfer
 
 struct dpde_handle {
@@ -103,7 +109,8 @@ struct dpde_handle {
         // blocks per SM), large (one block per SM)
         int scap_s[3] = {0, 0, 0}, ecap_s[3] = {0, 0, 0}, ccap_s[3] = {0, 0, 0}, scap_x[3] = {0, 0, 0};
         int grid_s[3] = {0, 0, 0}, grid_x[3] = {0, 0, 0};
-        bool ok = false;   // domains small enough for the level form
+        int stride = SSA_MAXLEV + 2;   // levels kept of a domain, + 2
+        bool ok = false;   // the level form is possible and expected to be the faster one
     } ssa_caps[2];
     int nsm = 152;
     // the persistent per-class SSA launch (ssa_mode 3): class offsets on the
@@ -111,6 +118,7 @@ struct dpde_handle {
     int* d_col_off[2] = {nullptr, nullptr};
     GridBarrier* d_bar = nullptr;
     long long wait_budget = 2000000000ll;
+    int cells_lcap = 16;      // particles staged by a warp of k_ssa_cells
     int ssa_group = 0;        // bricks per warp; 0 = dom_group_auto
     int dom_group_auto = 1;   // 32 / the largest class of a brick, in 1..SSA_GROUP_MAX
     ForceShape tile_shape{}, tile_shape_dense{};   // shared-memory shapes of the two force launches
@@ -268,6 +276,7 @@ void enqueue_ssa_levels(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T dt, 
     SsaLevels<T> V;
     V.lv_off = h->lv_off;
     V.lv_n = h->lv_n;
+    V.stride = K.stride;
     V.rec = reinterpret_cast<SsaRec<T>*>(h->fwd_g);   // (unused by this form: the forward entries' Gaussians)
     // counts: [0, 1] schedule tiers 1, 2; [2, 3] execution tiers 1, 2 of the
     // domains the regular schedule kept; [4, 5] execution tiers 1, 2 of those
@@ -278,19 +287,19 @@ void enqueue_ssa_levels(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T dt, 
     cudaMemsetAsync(cnt, 0, SSA_NLISTS * sizeof(int), st);
     auto sched_tiers = [&](cudaStream_t s) {
         for (int t = 1; t < 3; ++t)
-            k_ssa_sched<T><<<K.grid_s[t], SCHED_THREADS, ssa_sched_smem(K.scap_s[t], K.ecap_s[t], K.ccap_s[t]),
+            k_ssa_sched<T><<<K.grid_s[t], SCHED_THREADS, ssa_sched_smem(K.scap_s[t], K.ecap_s[t], K.ccap_s[t], K.stride),
                              s>>>(C, D, V, K.scap_s[t], K.ecap_s[t], K.ccap_s[t], 0, lst[t - 1], cnt + t - 1,
                                   t < 2 ? lst[t] : nullptr, t < 2 ? cnt + t : nullptr);
     };
     // execution tiers 1, 2 over the list at index l0 (tier 1) and l0 + 1 (tier 2)
     auto exec_tiers = [&](cudaStream_t s, int* first, int* nfirst, int l1) {
-        k_ssa_exec<T><<<K.grid_x[1], h->ssa_block + SSA_DRAW_THREADS, ssa_exec_smem<T>(K.scap_x[1]), s>>>(
+        k_ssa_exec<T><<<K.grid_x[1], h->ssa_block + SSA_DRAW_THREADS, ssa_exec_smem<T>(K.scap_x[1], K.stride), s>>>(
             C, D, V, K.scap_x[1], 0, first, nfirst, lst[l1], cnt + l1, dt, sqrt_dt);
-        k_ssa_exec<T><<<K.grid_x[2], h->ssa_block + SSA_DRAW_THREADS, ssa_exec_smem<T>(K.scap_x[2]), s>>>(
+        k_ssa_exec<T><<<K.grid_x[2], h->ssa_block + SSA_DRAW_THREADS, ssa_exec_smem<T>(K.scap_x[2], K.stride), s>>>(
             C, D, V, K.scap_x[2], 0, lst[l1], cnt + l1, nullptr, nullptr, dt, sqrt_dt);
     };
     auto sched_regular = [&](cudaStream_t s, int d0, int n) {
-        k_ssa_sched<T><<<n, SCHED_THREADS, ssa_sched_smem(K.scap_s[0], K.ecap_s[0], K.ccap_s[0]), s>>>(
+        k_ssa_sched<T><<<n, SCHED_THREADS, ssa_sched_smem(K.scap_s[0], K.ecap_s[0], K.ccap_s[0], K.stride), s>>>(
             C, D, V, K.scap_s[0], K.ecap_s[0], K.ccap_s[0], d0, nullptr, nullptr, lst[0], cnt);
     };
     auto exec_regular = [&](cudaStream_t s, int d0, int n) {
@@ -298,8 +307,8 @@ void enqueue_ssa_levels(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T dt, 
         // for each, so that no two share one while another is idle (the
         // deferred launches beside this one held SMs for a moment and packed
         // them: 125 domains in FP64, step 1461 us against the phases' 1015)
-        const size_t need = ssa_exec_smem<T>(K.scap_x[0]);
-        const size_t smem = n <= h->nsm ? std::max(need, std::min<size_t>(SSA_ALONE_SMEM, ssa_exec_smem<T>(K.scap_x[2]))) : need;
+        const size_t need = ssa_exec_smem<T>(K.scap_x[0], K.stride);
+        const size_t smem = n <= h->nsm ? std::max(need, std::min<size_t>(SSA_ALONE_SMEM, ssa_exec_smem<T>(K.scap_x[2], K.stride))) : need;
         k_ssa_exec<T><<<n, h->ssa_block + SSA_DRAW_THREADS, smem, s>>>(C, D, V, K.scap_x[0], d0, nullptr,
                                                                              nullptr, lst[2], cnt + 2, dt, sqrt_dt);
     };
@@ -378,7 +387,11 @@ void enqueue_ssa(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T dt, T sqrt_
     }
     for (int k = 0; k < NCOLOURS; ++k) {
         const int n = off[k + 1] - off[k];
-        if (n > 0)
+        if (n == 0) continue;
+        if (n <= CELLS_SM * h->nsm)
+            k_ssa_cells<T><<<n, 32, ssa_cells_smem<T>(h->cells_lcap), st>>>(C, h->col_cells[whole] + off[k], whole,
+                                                                          h->cells_lcap, dt, sqrt_dt);
+        else
             k_ssa_colour<T><<<ceil_div(n, h->ssa_block), h->ssa_block, ssa_smem_bytes(h->ssa_block), st>>>(
                 C, h->col_cells[whole] + off[k], n, dt, sqrt_dt);
     }
@@ -801,6 +814,9 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
     h->nbricks = (int)nbricks;
     h->nchunks = (int)chunk_rep.size();
     h->per_cell_max = per_cell_max;
+    // 1.6x the mean count of 14 cells, + 48, as far as 48 KB hold them
+    h->cells_lcap = (int)std::min(1.6 * 14.0 * per_cell_max + 48.0,
+                                  48.0 * 1024 / (double)(h->mixed ? ssa_cells_smem<float>(1) : ssa_cells_smem<double>(1))) & ~3;
     // neighbour-list capacity: 3x the mean neighbour count of the densest replica, + 32
     const double mean_nbr = 4.0 / 3.0 * M_PI * rho_max * P.r_cut * P.r_cut * P.r_cut;
     h->nbr_cap = (int)std::ceil(3.0 * mean_nbr) + 32;
@@ -914,11 +930,35 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
             for (const RepInfo& I : h->info)
                 biggest = std::max(biggest, t == 0 ? (double)I.n / (I.B[0] * I.B[1] * I.B[2]) : (double)I.n);
             const double M = ndom > 0 ? (double)N / ndom : 0.0;
+            // Whole replicas (DPDE_SSA): a block per replica level by level,
+            // or all cells of a class at once, class by class. Times in us
+            // per step of the largest replica, fitted to both forms at 300 to
+            // 20,000 particles of density 3 and 343 to 6,000 Lennard-Jones
+            // ones: levels ~ classes (4.5 + 0.075 m) with m maps a cell, a
+            // round of 64 maps at most a level; a class, its latency and m
+            // maps of its cells. (Mixed, levels / classes: 4,000 particles
+            // 422 / 739, 6,000 466 / 261, 8,000 928 / 576, 16,000 5849 / 830;
+            // LJ 343 523 / 2548.)
+            double level_us = 0.0, class_us = 1.0;
+            if (t == 1) {
+                int ncls = 0;
+                for (int k = 0; k < NCOLOURS; ++k) ncls += h->col_off[1][k + 1] > h->col_off[1][k];
+                double m = 0.0;
+                for (const RepInfo& I : h->info) m = std::max(m, I.n * e_pp / 1.15 / I.ncells);
+                const double maps = biggest * e_pp / 1.15, nlev = ncls * (4.5 + 0.075 * m);
+                if (n_replicas <= 1024 && nlev > 0.6 * SSA_MAXLEV)
+                    K.stride = (int)std::min<double>(SSA_MAXLEV_LONG, 1.5 * nlev + 64.0) + 2;
+                const size_t fixed = h->mixed ? ssa_exec_smem<float>(0, K.stride) : ssa_exec_smem<double>(0, K.stride);
+                level_us = (h->mixed ? 0.7 : 3.5) * std::max(nlev, maps / 64.0);
+                if (biggest > (double)((smem_big - fixed) / per)) level_us *= 1.4;   // state not in shared memory
+                if (maps > 0.88 * SSA_LOCAL_MAX || nlev > SSA_MAXLEV_LONG) level_us = INFINITY;   // no schedule
+                class_us = ncls * (h->mixed ? 6.0 + 0.28 * m : 28.0 + 2.05 * m);
+            }
             auto up16 = [](double x) { return ((int)std::ceil(x) + 15) / 16 * 16; };
             // entries that fit beside sc particles in ~200 KB of schedule
             auto ecap_fit = [&](int sc, int cc) {
                 return std::min(SSA_LOCAL_MAX,
-                                (int)((smem_big - (SSA_LV_STRIDE + 4 + cc) * sizeof(int)) / 2 - (2 * sc + 1)) / 16 * 16);
+                                (int)((smem_big - (K.stride + 4 + cc) * sizeof(int)) / 2 - (2 * sc + 1)) / 16 * 16);
             };
             // schedule: 1.3 M particles / 1.2 M e entries; 2.5 M / 6.25 M e (a
             // brick compressed 2.5-fold holds ~6x the entries) in ~96 KB; the
@@ -931,26 +971,26 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
             K.ccap_s[1] = K.scap_s[1] / 2;
             K.ecap_s[1] = std::min(ecap_fit(K.scap_s[1], K.ccap_s[1]), up16(6.25 * M * e_pp + 256));
             while (K.ecap_s[1] > K.ecap_s[0] &&
-                   ssa_sched_smem(K.scap_s[1], K.ecap_s[1], K.ccap_s[1]) > smem_big / 2)
+                   ssa_sched_smem(K.scap_s[1], K.ecap_s[1], K.ccap_s[1], K.stride) > smem_big / 2)
                 K.ecap_s[1] = std::max(K.ecap_s[0], K.ecap_s[1] * 7 / 8 / 16 * 16);
             K.scap_s[2] = 16384;
             K.ccap_s[2] = 0;
             K.ecap_s[2] = ecap_fit(K.scap_s[2], 0);
             // execution: M + 5 sqrt(M) + 32 particles; 2.5 M in <= 96 KB; ~200 KB
-            const int xfit = (int)((smem_big - (h->mixed ? ssa_exec_smem<float>(0) : ssa_exec_smem<double>(0))) / per) & ~3;
+            const int xfit = (int)((smem_big - (h->mixed ? ssa_exec_smem<float>(0, K.stride) : ssa_exec_smem<double>(0, K.stride))) / per) & ~3;
             K.scap_x[0] = std::min(xfit, ((int)std::ceil(M + 5.0 * std::sqrt(M) + 32) + 31) / 32 * 32);
             K.scap_x[1] = std::max(K.scap_x[0], std::min(xfit / 2 & ~3, ((int)std::ceil(2.5 * M + 64) + 31) / 32 * 32));
             K.scap_x[2] = xfit;
             const size_t smem_sm = 227 * 1024;
             K.grid_s[0] = ndom;
             K.grid_s[1] = h->nsm * std::max<int>(1, (int)(smem_sm / (ssa_sched_smem(K.scap_s[1], K.ecap_s[1],
-                                                                                      K.ccap_s[1]) + 1024)));
+                                                                                      K.ccap_s[1], K.stride) + 1024)));
             K.grid_s[2] = h->nsm;
             K.grid_x[0] = ndom;
-            const size_t xs1 = h->mixed ? ssa_exec_smem<float>(K.scap_x[1]) : ssa_exec_smem<double>(K.scap_x[1]);
+            const size_t xs1 = h->mixed ? ssa_exec_smem<float>(K.scap_x[1], K.stride) : ssa_exec_smem<double>(K.scap_x[1], K.stride);
             K.grid_x[1] = h->nsm * std::max<int>(1, std::min<int>(8, (int)(smem_sm / (xs1 + 1024))));
             K.grid_x[2] = h->nsm;
-            K.ok = biggest <= 16384.0;
+            K.ok = biggest <= 16384.0 && level_us <= class_us;
         }
     }
     auto bail = [&](cudaError_t e, const char* what) {
@@ -1070,15 +1110,15 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
     CKC(cudaMemcpy(h->rdom_off, rdom_off.data(), sizeof(int) * rdom_off.size(), cudaMemcpyHostToDevice));
     CKC(cudaMemcpy(h->rdom_cell0, rdom_cell0.data(), sizeof(int) * rdom_cell0.size(), cudaMemcpyHostToDevice));
     h->ndom_max = std::max(1, std::max(h->nbricks, h->R));
-    CKC(cudaMalloc(&h->lv_off, sizeof(int) * (size_t)h->ndom_max * SSA_LV_STRIDE));
+    CKC(cudaMalloc(&h->lv_off, sizeof(int) * std::max((size_t)h->nbricks * h->ssa_caps[0].stride, (size_t)h->R * h->ssa_caps[1].stride)));
     CKC(cudaMalloc(&h->lv_n, sizeof(int) * (size_t)h->ndom_max));
     CKC(cudaMalloc(&h->ssa_defer, sizeof(int) * (SSA_NLISTS + SSA_NLISTS * (size_t)h->ndom_max)));
     {
         size_t ms = 0, mx = 0;
         for (const auto& K : h->ssa_caps)
             for (int t = 0; t < 3; ++t) {
-                ms = std::max(ms, ssa_sched_smem(K.scap_s[t], K.ecap_s[t], K.ccap_s[t]));
-                mx = std::max(mx, h->mixed ? ssa_exec_smem<float>(K.scap_x[t]) : ssa_exec_smem<double>(K.scap_x[t]));
+                ms = std::max(ms, ssa_sched_smem(K.scap_s[t], K.ecap_s[t], K.ccap_s[t], K.stride));
+                mx = std::max(mx, h->mixed ? ssa_exec_smem<float>(K.scap_x[t], K.stride) : ssa_exec_smem<double>(K.scap_x[t], K.stride));
             }
         const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
         if (h->mixed) {

@@ -38,8 +38,11 @@
 
 namespace dpde {
 
-constexpr int SSA_MAXLEV = 1023;         // levels of one domain kept by the schedule
-constexpr int SSA_LV_STRIDE = SSA_MAXLEV + 2;
+// levels of one domain kept by the schedule: 1023, and up to 4095 for whole
+// replicas with long rows (Lennard-Jones: 343 particles have ~830 levels,
+// 1,000 ~1,120; a schedule that did not fit ran its domain in colour order on
+// one block, 11.5 ms a step against 0.8 now)
+constexpr int SSA_MAXLEV = 1023, SSA_MAXLEV_LONG = 4095;
 constexpr int SCHED_THREADS = 128;
 constexpr int SSA_ROW_BATCH = 8;        // entries of a row taken together
 constexpr int SSA_LEV_BATCH = 8;        // ... by the level walk
@@ -62,7 +65,7 @@ struct SsaDomains {
 };
 
 // The level schedule of every domain: per domain the record offsets of its
-// levels (lv_off[d * SSA_LV_STRIDE + l], l = 0..nlev, records of level l in
+// levels (lv_off[d * stride + l], l = 0..nlev, records of level l in
 // [lv_off[l], lv_off[l + 1])), its level count (lv_n[d]: nlev >= 0 from the
 // regular launch, -3 - nlev from a deferred one, -1 no schedule (executed
 // along the colour order), SSA_PENDING = -2 deferred and not yet scheduled),
@@ -80,22 +83,23 @@ struct SsaLevels {
     int* lv_off;
     int* lv_n;
     SsaRec<T>* rec;
+    int stride;   // the most levels + 2
 };
 
-// shared bytes of k_ssa_sched for scap particles, ecap entries and ccap
-// cells: cnt (counters of levels 0..SSA_MAXLEV + 1) | cr[ccap] (the domain's
+// shared bytes of k_ssa_sched for scap particles, ecap entries, ccap cells and
+// a level stride: cnt (counters of levels 0..stride - 1, one more) | cr[ccap] (the domain's
 // cells in class order: local start | count << 16) | rowoff[scap + 1] |
 // L[scap] | ent[ecap] (16-bit)
-__host__ __device__ constexpr size_t ssa_sched_smem(int scap, int ecap, int ccap) {
-    return (size_t)(SSA_LV_STRIDE + 1 + ccap) * sizeof(int) +
+__host__ __device__ constexpr size_t ssa_sched_smem(int scap, int ecap, int ccap, int stride) {
+    return (size_t)(stride + 1 + ccap) * sizeof(int) +
            (((size_t)(2 * scap + 1 + ecap) * 2 + 15) / 16) * 16;
 }
 // shared bytes of k_ssa_exec for scap staged particles (a multiple of 4): p |
 // drawn (G, w) of the chunks held | eps | id | their records | level starts
 template <class T>
-__host__ __device__ constexpr size_t ssa_exec_smem(int scap) {
+__host__ __device__ constexpr size_t ssa_exec_smem(int scap, int stride) {
     return (size_t)scap * (sizeof(vec_t<T>) + sizeof(eps_t<T>) + sizeof(uint32_t)) +
-           (size_t)SSA_RING * SSA_CHUNK * (sizeof(vec_t<T>) + sizeof(uint32_t)) + (size_t)SSA_LV_STRIDE * 2 + 16;
+           (size_t)SSA_RING * SSA_CHUNK * (sizeof(vec_t<T>) + sizeof(uint32_t)) + (size_t)stride * 2 + 16;
 }
 
 // slot range [sb, se) of domain d
@@ -146,7 +150,7 @@ __device__ __forceinline__ void ssa_rows(int nb, const unsigned short* rowoff, c
 }
 
 // One domain's schedule on the calling block. Returns false (nothing written)
-// when the domain exceeds scap particles, ecap entries or SSA_MAXLEV levels.
+// when the domain exceeds scap particles, ecap entries or the levels kept.
 template <class T>
 __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const SsaLevels<T>& V, int d, int scap,
                                  int ecap, int ccap, bool deferred, unsigned char* smem) {
@@ -159,7 +163,7 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
     const int tid = threadIdx.x;
     if (nb > scap || nb > SSA_LOCAL_MAX) return false;
     int* cnt = reinterpret_cast<int*>(smem);
-    unsigned int* cr = reinterpret_cast<unsigned int*>(cnt + SSA_LV_STRIDE + 1);
+    unsigned int* cr = reinterpret_cast<unsigned int*>(cnt + V.stride + 1);
     unsigned short* rowoff = reinterpret_cast<unsigned short*>(cr + ccap);
     unsigned short* L = rowoff + scap + 1;
     unsigned short* ent = L + scap;    // partner (local slot) of each entry, then its level
@@ -167,7 +171,7 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
         s_flag = 0;
         s_nlev = 0;
     }
-    for (int l = tid; l <= SSA_LV_STRIDE; l += blockDim.x) cnt[l] = 0;
+    for (int l = tid; l <= V.stride; l += blockDim.x) cnt[l] = 0;
     const int* off = D.off + (size_t)d * (NCOLOURS + 1);
     for (int k = tid; k <= NCOLOURS; k += blockDim.x) s_off[k] = __ldg(off + k);
     __syncthreads();
@@ -216,8 +220,7 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
     for (int k = 0; k < NCOLOURS; ++k) {
         const int k0 = s_off[k], k1 = s_off[k + 1];
         if (k1 == k0) continue;   // uniform over the block
-        for (int u = k0 + tid; u < k1; u += blockDim.x) {
-            int i, iend;
+        auto cell_range = [&](int u, int& i, int& iend) {
             if (cstaged) {
                 const unsigned int v = cr[u - cbase];
                 i = (int)(v & 0xffffu);
@@ -227,6 +230,10 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
                 i = C.start[c] - sb;
                 iend = C.start[c + 1] - sb;
             }
+        };
+        for (int u = k0 + tid; u < k1; u += blockDim.x) {
+            int i, iend;
+            cell_range(u, i, iend);
             int e = i < iend ? rowoff[i] : 0;
             for (; i < iend; ++i) {
                 const int end = rowoff[i + 1];
@@ -260,11 +267,11 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
     atomicMax(&s_nlev, mylev);
     __syncthreads();
     const int nlev = s_nlev;
-    if (nlev > SSA_MAXLEV) return false;
+    if (nlev > V.stride - 2) return false;
     // 4. records sorted by level: counts, offsets, scatter
     for (int e = tid; e < E; e += blockDim.x) atomicAdd(cnt + ent[e], 1);
     __syncthreads();
-    int* lvo = V.lv_off + (size_t)d * SSA_LV_STRIDE;
+    int* lvo = V.lv_off + (size_t)d * V.stride;
     if (tid < 32) {
         // exclusive scan of the counts of levels 1..nlev: lvo[l - 1] = start
         // of level l, lvo[nlev] = E; the counters become the cursors
@@ -521,7 +528,7 @@ __device__ void ssa_exec_domain(const Ctx<T>& C, const SsaDomains& D, const SsaL
         if (threadIdx.x == 0) defer[atomicAdd(ndefer, 1)] = d;
         return;
     }
-    const int* lvo = V.lv_off + (size_t)d * SSA_LV_STRIDE;
+    const int* lvo = V.lv_off + (size_t)d * V.stride;
     for (int l = threadIdx.x; l <= nlev; l += blockDim.x) lvs[l] = (unsigned short)lvo[l];
     if (nb > scap) {
         __syncthreads();
