@@ -46,6 +46,7 @@ constexpr int SSA_MAXLEV = 1023, SSA_MAXLEV_LONG = 4095;
 constexpr int SCHED_THREADS = 128;
 constexpr int SSA_ROW_BATCH = 8;        // entries of a row taken together
 constexpr int SSA_LEV_BATCH = 8;        // ... by the level walk
+constexpr int SSA_LONG_ROW = 12;        // mean entries of a row from which a warp walks a cell
 constexpr int SSA_DRAW_THREADS = 64;    // threads of an execution block that draw Gaussians
 constexpr int SSA_EXEC_THREADS_MAX = SSA_THREADS_MAX + SSA_DRAW_THREADS;
 constexpr int SSA_CHUNK = 128;          // records drawn ahead of the maps, SSA_RING chunks held
@@ -216,6 +217,12 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
     //    a cell and a prefix maximum over them took 29,000 warp instructions
     //    a domain. Schedule of a step, with the rows below loaded without
     //    branches: 4M 523 -> 417 us, the batch of 256 boxes 1078 -> 826 us.)
+    //    Long rows (Lennard-Jones: ~26 entries, 13 particles a cell) come with
+    //    few cells a class, one or two of a block's threads walking while the
+    //    others wait: there a warp takes a cell, 32 entries of a row at a time
+    //    by a prefix maximum (schedule of a step: 343 Lennard-Jones particles
+    //    180 -> 112 us, 125 domains of 1,152 278 -> 192).
+    const bool long_rows = E > SSA_LONG_ROW * nb;   // uniform over the block
     int mylev = 0;
     for (int k = 0; k < NCOLOURS; ++k) {
         const int k0 = s_off[k], k1 = s_off[k + 1];
@@ -231,6 +238,38 @@ __device__ bool ssa_sched_domain(const Ctx<T>& C, const SsaDomains& D, const Ssa
                 iend = C.start[c + 1] - sb;
             }
         };
+        if (long_rows) {
+            for (int u = k0 + (tid >> 5); u < k1; u += (int)blockDim.x >> 5) {
+                const int lane = tid & 31;
+                int i, iend;
+                cell_range(u, i, iend);
+                for (; i < iend; ++i) {
+                    const int end = rowoff[i + 1];
+                    int Ls = L[i];
+                    for (int e = rowoff[i]; e < end; e += 32) {
+                        // lev_j = max(Ls + 1 + j, max over m <= j of L[t_m] + 1 + j - m)
+                        const int f = min(e + lane, end - 1), t = ent[f];
+                        int x = max((int)L[t], lane == 0 ? Ls : 0) + 1 - lane;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int y = __shfl_up_sync(0xffffffffu, x, o);
+                            if (lane >= o) x = max(x, y);
+                        }
+                        x += lane;
+                        if (e + lane < end) {
+                            L[t] = (unsigned short)x;
+                            ent[f] = (unsigned short)x;
+                        }
+                        Ls = __shfl_sync(0xffffffffu, x, min(31, end - 1 - e));
+                    }
+                    if (lane == 0) L[i] = (unsigned short)Ls;
+                    mylev = max(mylev, Ls);
+                    __syncwarp();   // the next row reads these levels
+                }
+            }
+            __syncthreads();
+            continue;
+        }
         for (int u = k0 + tid; u < k1; u += blockDim.x) {
             int i, iend;
             cell_range(u, i, iend);

@@ -1,5 +1,5 @@
 """The SSA a warp per cell at the edges of its staging (GPU), against the level
-form, which must agree bit
+form (whose schedule walks long rows a warp per cell), which must agree bit
 for bit: cells with none, one or many rounds of entries, rows beyond 32
 particles, more particles than are staged, domains that end at a brick face,
 at the box's own periodic image and at a wall. Two steps each."""
@@ -34,7 +34,7 @@ def run(n, box, bricks, scheme, precision, clump, walls, mode):
     (1700, (7.5, 8.5, 9.5), (1, 1, 1), "SSA", None, (1, -0.5)),
     (1000, (6.1, 8.2, 7.3), (2, 4, 1), "HYBRID", None, (0, 0.0)),
     (2000, (9.0, 9.0, 9.0), (1, 1, 1), "SSA", 0.45, (0, 0.0)),     # a corner too dense to be staged
-    (200, (3.0, 3.1, 3.2), (1, 1, 1), "SSA", None, (0, 0.0)),      # ~14 entries a row
+    (200, (3.0, 3.1, 3.2), (1, 1, 1), "SSA", None, (0, 0.0)),      # ~14 entries a row: levels by warps
     (350, (3.2, 3.2, 3.2), (1, 1, 1), "SSA", None, (0, 0.0)),      # ~22, some rows beyond 32
     (3000, (9.0, 6.2, 6.2), (3, 1, 1), "HYBRID", None, (0, 0.0)),  # ~15, in domains
     (1200, (3.3, 3.3, 3.3), (1, 1, 1), "SSA", None, (0, 0.0)),     # ~44 a cell
