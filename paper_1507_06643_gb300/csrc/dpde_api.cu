@@ -419,7 +419,7 @@ void enqueue_step(dpde_handle* h, cudaStream_t st, double dt_d, int scheme) {
     }
     phase(h, st, DPDE_PHASE_SWEEP2, 0);
     if (scheme == DPDE_SER || scheme == DPDE_HYBRID) k_ser_sweep2<T><<<ceil_div(h->N, SER_THREADS), SER_THREADS, 0, st>>>(C);
-    else if (scheme == DPDE_SEM) k_sem<T><<<nb, h->block, 0, st>>>(C, dt, sqrt_dt);
+    else if (scheme == DPDE_SEM) k_sem<T><<<ceil_div(h->N, SER_THREADS), SER_THREADS, 0, st>>>(C, dt, sqrt_dt);
     else k_copy_back<T><<<nb, h->block, 0, st>>>(C);
     phase(h, st, DPDE_PHASE_SWEEP2, 1);
     if (h->project) {

@@ -538,6 +538,26 @@ __device__ __forceinline__ T3<T> ser_dp(const Ctx<T>& C, int j, T w, uint32_t st
                  A * ((pi.z - pj.z) * C.inv_m) + Bn * G.z};
 }
 
+// the entries [c0, c0 + win) of the warp's flat list, a lane per owner i with
+// four loads in flight (past the end the last one again)
+template <class T>
+__device__ __forceinline__ void ser_window(const Ctx<T>& C, const WarpEntries& W, int i, int c0, int win, ListEnt<T>* ent) {
+    const int excl = W.incl - W.nn, k1 = min(W.nn, c0 + win - excl);
+    const ListEnt<T>* row = C.nbr + i;
+    for (int k = max(0, c0 - excl); k < k1; k += 4) {
+        ListEnt<T> v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = row[(size_t)min(k + u, k1 - 1) * (size_t)C.N];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (k + u < k1) {
+                v[u].j = (int)pack_owner(v[u].j, W.lane);
+                ent[excl + k + u - c0] = v[u];
+            }
+    }
+    __syncwarp();
+}
+
 // first sweep: delta p_i = sum_j delta p_ij (Eq. SER_p). Each delta p_ij is
 // also written, with its partner and owner, into the forward-entry buffer
 // fwd_g (free once the SSA part of the step is done), the entries of a warp's
@@ -553,27 +573,10 @@ __global__ void __launch_bounds__(SER_THREADS) k_ser_sweep1(Ctx<T> C, T dt, T sq
     const WarpEntries W = warp_entries(i < C.N ? C.nbr_n[i] : 0);
     const uint32_t step = (uint32_t)*C.step;
     const T sdt = C.sigma * sqrt_dt;
-    const size_t N = (size_t)C.N;
-    const int excl = W.incl - W.nn;
     vec_t<T>* const out_g = C.fwd_g + (size_t)base * C.nbr_cap;
     T ax = 0, ay = 0, az = 0;
     for (int c0 = 0; c0 < W.total; c0 += WIN) {
-        // my entries of the window, four loads in flight (past the end the
-        // last one again)
-        const int k1 = min(W.nn, c0 + WIN - excl);
-        const ListEnt<T>* row = C.nbr + i;
-        for (int k = max(0, c0 - excl); k < k1; k += 4) {
-            ListEnt<T> v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = row[(size_t)min(k + u, k1 - 1) * N];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (k + u < k1) {
-                    v[u].j = (int)pack_owner(v[u].j, W.lane);
-                    ent[excl + k + u - c0] = v[u];
-                }
-        }
-        __syncwarp();
+        ser_window(C, W, i, c0, WIN, ent);
         const int end = min(W.total, c0 + WIN);
         for (int f0 = c0; f0 < end; f0 += 32) {
             const int f = f0 + W.lane;
@@ -685,38 +688,64 @@ __global__ void __launch_bounds__(SER_THREADS) k_ser_sweep2(Ctx<T> C) {
 
 // ---------------------------------------------------------------------------
 // SEM, Eq. (SEM_fd): one sweep, Euler-Maruyama on p and eps. B -> A.
+//
+// Issue-bound, most of it the draw: a thread per particle drew for the longest
+// list of its warp (20 entries of 12.6 at density 3). The entries are spread
+// over the lanes as in the SER sweeps, their increments left in shared memory
+// and summed by the owner in list order (250,047 particles 41.5 -> 39.8 us,
+// 1.4 waves of blocks).
 // ---------------------------------------------------------------------------
 template <class T>
-__global__ void k_sem(Ctx<T> C, T dt, T sqrt_dt) {
+__global__ void __launch_bounds__(SER_THREADS) k_sem(Ctx<T> C, T dt, T sqrt_dt) {
+    constexpr int WIN = SERWIN_BYTES / 2 / (int)sizeof(ListEnt<T>);
+    __shared__ ListEnt<T> win[SER_THREADS / 32][WIN];
+    __shared__ vec_t<T> inc[SER_THREADS / 32][WIN];
+    ListEnt<T>* const ent = win[threadIdx.x >> 5];
+    vec_t<T>* const val = inc[threadIdx.x >> 5];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= C.N) return;
-    const int rep = C.rep_of_slot[i];
-    const RepInfo& R = C.reps[rep];
-    const vec_t<T> pi = C.pB[i];
-    const uint32_t idi = C.idB[i];
+    const int base = i - (int)(threadIdx.x & 31);
+    const WarpEntries W = warp_entries(i < C.N ? C.nbr_n[i] : 0);
     const uint32_t step = (uint32_t)*C.step;
-    const int nn = C.nbr_n[i];
     const T d_sig2_m = T(3) * C.sigma * C.sigma * C.inv_m;
     const T sdt = C.sigma * sqrt_dt;
+    const int excl = W.incl - W.nn;
     T ax = 0, ay = 0, az = 0, de = 0;
-    for (int k = 0; k < nn; ++k) {
-        const ListEnt<T> en = C.nbr[(size_t)k * C.N + i];
-        const int j = en.j;
-        const T w = en.w;
-        const vec_t<T> pj = C.pB[j];
-        const T chi = w * w;
-        const T gam = C.sig2_4 * (pi.w + pj.w);
-        const T3<T> G = pair_gauss<T>(C.seed, step, (uint32_t)rep, idi, C.idB[j]);
-        const T vx = (pi.x - pj.x) * C.inv_m;
-        const T vy = (pi.y - pj.y) * C.inv_m;
-        const T vz = (pi.z - pj.z) * C.inv_m;
-        const T A = -gam * chi * dt, Bn = sdt * w;
-        ax += A * vx + Bn * G.x;
-        ay += A * vy + Bn * G.y;
-        az += A * vz + Bn * G.z;
-        de += T(0.5) * (gam * (vx * vx + vy * vy + vz * vz) - d_sig2_m) * chi * dt -
-              T(0.5) * Bn * (vx * G.x + vy * G.y + vz * G.z);
+    for (int c0 = 0; c0 < W.total; c0 += WIN) {
+        ser_window(C, W, i, c0, WIN, ent);
+        const int end = min(W.total, c0 + WIN);
+        for (int f = c0 + W.lane; f < end; f += 32) {
+            const ListEnt<T> en = ent[f - c0];
+            const int io = base + owner_of((uint32_t)en.j), j = partner_of((uint32_t)en.j);
+            const T w = en.w;
+            const vec_t<T> pi = C.pB[io], pj = C.pB[j];
+            const T chi = w * w;
+            const T gam = C.sig2_4 * (pi.w + pj.w);
+            const T3<T> G = pair_gauss<T>(C.seed, step, (uint32_t)C.rep_of_slot[io], C.idB[io], C.idB[j]);
+            const T vx = (pi.x - pj.x) * C.inv_m;
+            const T vy = (pi.y - pj.y) * C.inv_m;
+            const T vz = (pi.z - pj.z) * C.inv_m;
+            const T A = -gam * chi * dt, Bn = sdt * w;
+            vec_t<T> v;
+            v.x = A * vx + Bn * G.x;
+            v.y = A * vy + Bn * G.y;
+            v.z = A * vz + Bn * G.z;
+            v.w = T(0.5) * (gam * (vx * vx + vy * vy + vz * vz) - d_sig2_m) * chi * dt -
+                  T(0.5) * Bn * (vx * G.x + vy * G.y + vz * G.z);
+            val[f - c0] = v;
+        }
+        __syncwarp();
+        for (int f = max(c0, excl); f < min(W.incl, end); ++f) {
+            const vec_t<T> v = val[f - c0];
+            ax += v.x;
+            ay += v.y;
+            az += v.z;
+            de += v.w;
+        }
+        __syncwarp();   // the window has been read
     }
+    if (i >= C.N) return;
+    const RepInfo& R = C.reps[C.rep_of_slot[i]];
+    const vec_t<T> pi = C.pB[i];
     vec_t<T> pn = pi;
     pn.x = pi.x + ax; pn.y = pi.y + ay; pn.z = pi.z + az;
     const eps_t<T> en = eps_add(C.eB[i], de);
