@@ -217,8 +217,10 @@ void enqueue_sort(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T half_dt, T
     phase(h, st, DPDE_PHASE_SCAN, 0);
     const int ntile = ceil_div(h->ncells, SCAN_TILE);
     k_scan_local<<<ntile, SCAN_THREADS, 0, st>>>(h->cnt, h->start, h->bsum, h->ncells);
-    k_scan_bsums<<<1, 1024, 0, st>>>(h->bsum, ntile);
-    k_scan_add<<<ceil_div(h->ncells, 256), 256, 0, st>>>(h->start, h->bsum, h->ncells, h->N);
+    const bool scanned = ntile > SCAN_SELF;
+    if (scanned) k_scan_bsums<<<1, 1024, 0, st>>>(h->bsum, ntile);
+    k_scan_add<<<ceil_div(h->ncells, SCAN_ADD_THREADS), SCAN_ADD_THREADS, 0, st>>>(
+        h->start, h->bsum, h->ncells, h->N, scanned, h->defer + h->ntiles, h->ssa_defer, SSA_NLISTS);
     phase(h, st, DPDE_PHASE_SCAN, 1);
     phase(h, st, DPDE_PHASE_GATHER, 0);
     k_scatter<T><<<nb + ceil_div(h->frames.n, h->block / 32), h->block, 0, st>>>(C, h->frames, nb);
@@ -239,7 +241,7 @@ void enqueue_force(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T half_dt, 
     const dim3 g(h->ntiles), blk(32 * h->tile_warps), gd(h->ndense_blocks), bd(32 * h->tile_warps_dense);
     const size_t sm = force_smem<T>(S0, h->tile_warps), smd = force_smem<T>(S1, h->tile_warps_dense);
     int* cnt = h->defer + h->ntiles;
-    cudaMemsetAsync(cnt, 0, sizeof(int), st);
+    if (list == LIST_OBS) cudaMemsetAsync(cnt, 0, sizeof(int), st);   // (else cleared by the sort before it)
 #define DPDE_FORCE(LMV)                                                                                           \
     k_force_tile<T, LMV><<<g, blk, sm, st>>>(C, h->tile_org, h->tile_dim, half_dt, kick, S0,                      \
                                              h->frames, h->defer, cnt);                                           \
@@ -280,11 +282,10 @@ void enqueue_ssa_levels(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T dt, 
     V.rec = reinterpret_cast<SsaRec<T>*>(h->fwd_g);   // (unused by this form: the forward entries' Gaussians)
     // counts: [0, 1] schedule tiers 1, 2; [2, 3] execution tiers 1, 2 of the
     // domains the regular schedule kept; [4, 5] execution tiers 1, 2 of those
-    // it deferred; then the lists
+    // it deferred; then the lists (the sort has cleared the counts)
     int* cnt = h->ssa_defer;
     int* lst[SSA_NLISTS];
     for (int k = 0; k < SSA_NLISTS; ++k) lst[k] = cnt + SSA_NLISTS + (size_t)k * h->ndom_max;
-    cudaMemsetAsync(cnt, 0, SSA_NLISTS * sizeof(int), st);
     auto sched_tiers = [&](cudaStream_t s) {
         for (int t = 1; t < 3; ++t)
             k_ssa_sched<T><<<K.grid_s[t], SCHED_THREADS, ssa_sched_smem(K.scap_s[t], K.ecap_s[t], K.ccap_s[t], K.stride),
