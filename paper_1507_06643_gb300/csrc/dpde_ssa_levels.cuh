@@ -71,9 +71,12 @@ struct SsaDomains {
 // regular launch, -3 - nlev from a deferred one, -1 no schedule (executed
 // along the colour order), SSA_PENDING = -2 deferred and not yet scheduled),
 // and the records, domain d's at [slot0(d) * cap, ...): (s_local | t_local
-// << 16) and the weight w, one 8- or 16-byte word. The execution's regular
-// launch, which may run beside the schedule's deferred launches, takes only
-// lv_n >= -1, so it never reads a schedule that is still being written.
+// << 16) and the weight w, one 8- or 16-byte word. Every domain with lv_n < 0
+// is on the list of those the regular schedule deferred and is executed from
+// that list, by the deferred launches. The execution's regular launch, which
+// may run beside them and beside the schedule's deferred launches, takes only
+// lv_n >= 0: no domain is executed twice, and no schedule is read that is
+// still being written.
 template <class T> struct __align__(2 * sizeof(T)) SsaRec {
     uint32_t st;
     T w;
@@ -539,7 +542,8 @@ __device__ void ssa_exec_classes(const Ctx<T>& C, const SsaDomains& D, int d, in
 
 // One domain on the calling block: staged in shared memory when it fits in
 // scap slots, else deferred (defer given) or run on global memory (defer ==
-// nullptr). The regular launch skips a domain whose schedule was deferred.
+// nullptr). The regular launch skips the domains the regular schedule
+// deferred, whether or not a later launch could schedule them.
 template <class T>
 __device__ void ssa_exec_domain(const Ctx<T>& C, const SsaDomains& D, const SsaLevels<T>& V, int d, int scap,
                                 bool regular, int* defer, int* ndefer, int nmap, T dt, T sqrt_dt, unsigned char* smem) {
@@ -549,9 +553,9 @@ __device__ void ssa_exec_domain(const Ctx<T>& C, const SsaDomains& D, const SsaL
     if (nb == 0) return;
     const int v = V.lv_n[d];
     const int rep = C.rep_of_cell[D.cell0[d]];
-    // deferred by the regular schedule: scheduled and executed by the deferred
-    // launches (perhaps running beside this one)
-    if (regular && v <= SSA_PENDING) return;
+    // deferred by the regular schedule: scheduled (or left without a schedule)
+    // and executed by the deferred launches, perhaps running beside this one
+    if (regular && v < 0) return;
     const int nlev = ssa_nlev(v);
     if (nlev < 0) {   // no schedule, even with the largest capacities: the colour order itself
         ssa_exec_classes(C, D, d, rep, dt, sqrt_dt);
