@@ -45,7 +45,12 @@ struct GraphKey {
 
 }  // namespace
 
-constexpr size_t FORCE_SMEM_MAX = 200 * 1024;   // dynamic shared memory of a force block, at most
+// Dynamic shared memory of a block of the force pass, of the SSA's schedule and
+// of its execution, at most. A kernel's limit is an attribute of the function,
+// which all handles of a process share: every handle sets it to the same value.
+constexpr size_t FORCE_SMEM_MAX = 200 * 1024;
+constexpr size_t SSA_SMEM_FIT = 200 * 1024;     // what the largest capacities are fitted to,
+constexpr size_t SSA_SMEM_MAX = SSA_SMEM_FIT + 1024;   // up to the arrays' rounding
 constexpr size_t SSA_ALONE_SMEM = 116 * 1024;   // one such block per SM
 // Cells of a colour class per SM up to which a warp takes a cell: its time is
 // that of the longest cell, ~10 us, until the warps fill the chip (SSA step at
@@ -569,6 +574,32 @@ void free_all(dpde_handle* h) {
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 
+// Lifts the limits on dynamic shared memory of the kernels that take more than
+// the default 48 KB.
+template <class T>
+cudaError_t allow_smem() {
+    const std::pair<const void*, size_t> limit[] = {
+        {(const void*)k_force_tile<T, LIST_NONE>, FORCE_SMEM_MAX},
+        {(const void*)k_force_tile<T, LIST_ALL>, FORCE_SMEM_MAX},
+        {(const void*)k_force_tile<T, LIST_CROSS>, FORCE_SMEM_MAX},
+        {(const void*)k_force_tile<T, LIST_FWD>, FORCE_SMEM_MAX},
+        {(const void*)k_force_tile<T, LIST_OBS>, FORCE_SMEM_MAX},
+        {(const void*)k_force_tile_dense<T, LIST_NONE>, FORCE_SMEM_MAX},
+        {(const void*)k_force_tile_dense<T, LIST_ALL>, FORCE_SMEM_MAX},
+        {(const void*)k_force_tile_dense<T, LIST_CROSS>, FORCE_SMEM_MAX},
+        {(const void*)k_force_tile_dense<T, LIST_FWD>, FORCE_SMEM_MAX},
+        {(const void*)k_force_tile_dense<T, LIST_OBS>, FORCE_SMEM_MAX},
+        {(const void*)k_ssa_sched<T>, SSA_SMEM_MAX},
+        {(const void*)k_ssa_exec<T>, SSA_SMEM_MAX},
+        {(const void*)k_ssa_domains<T>, (size_t)SSA_DOMAIN_SMEM}};
+    for (const auto& l : limit) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(l.first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.second);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // Force tiles: frame tiles of `edge` cells over every replica, each cut into
 // work tiles of wx x wy x wz cells (the tiles of the launch).
 int set_tiles(dpde_handle* h, int edge) {
@@ -640,7 +671,7 @@ int set_tiles(dpde_handle* h, int edge) {
         return S;
     };
     const ForceShape S0 = capped(1.08 * mean_halo() + 64.0), S1 = capped(2.5 * mean_halo() + 128.0);
-    const size_t smem = bytes(S0), smem_dense = bytes(S1, 1.7);
+    const size_t smem_dense = bytes(S1, 1.7);
     std::vector<int4> torg, tdim, forg;
     for (int r = 0; r < h->R; ++r) {
         const RepInfo& I = h->info[r];
@@ -678,31 +709,6 @@ int set_tiles(dpde_handle* h, int edge) {
     CK(h, cudaMemset(h->frame_rel, 0, std::max<size_t>(1, forg.size())));
     CK(h, cudaMemcpy(h->tile_org, torg.data(), sizeof(int4) * torg.size(), cudaMemcpyHostToDevice));
     CK(h, cudaMemcpy(h->tile_dim, tdim.data(), sizeof(int4) * tdim.size(), cudaMemcpyHostToDevice));
-    const int sm = (int)smem, smd = (int)smem_dense;
-    const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if (h->mixed) {
-        CK(h, cudaFuncSetAttribute(k_force_tile<float, LIST_NONE>, A, sm));
-        CK(h, cudaFuncSetAttribute(k_force_tile<float, LIST_ALL>, A, sm));
-        CK(h, cudaFuncSetAttribute(k_force_tile<float, LIST_CROSS>, A, sm));
-        CK(h, cudaFuncSetAttribute(k_force_tile<float, LIST_FWD>, A, sm));
-        CK(h, cudaFuncSetAttribute(k_force_tile_dense<float, LIST_NONE>, A, smd));
-        CK(h, cudaFuncSetAttribute(k_force_tile_dense<float, LIST_ALL>, A, smd));
-        CK(h, cudaFuncSetAttribute(k_force_tile_dense<float, LIST_CROSS>, A, smd));
-        CK(h, cudaFuncSetAttribute(k_force_tile_dense<float, LIST_FWD>, A, smd));
-        CK(h, cudaFuncSetAttribute(k_force_tile<float, LIST_OBS>, A, (int)FORCE_SMEM_MAX));
-        CK(h, cudaFuncSetAttribute(k_force_tile_dense<float, LIST_OBS>, A, (int)FORCE_SMEM_MAX));
-    } else {
-        CK(h, cudaFuncSetAttribute(k_force_tile<double, LIST_NONE>, A, sm));
-        CK(h, cudaFuncSetAttribute(k_force_tile<double, LIST_ALL>, A, sm));
-        CK(h, cudaFuncSetAttribute(k_force_tile<double, LIST_CROSS>, A, sm));
-        CK(h, cudaFuncSetAttribute(k_force_tile<double, LIST_FWD>, A, sm));
-        CK(h, cudaFuncSetAttribute(k_force_tile_dense<double, LIST_NONE>, A, smd));
-        CK(h, cudaFuncSetAttribute(k_force_tile_dense<double, LIST_ALL>, A, smd));
-        CK(h, cudaFuncSetAttribute(k_force_tile_dense<double, LIST_CROSS>, A, smd));
-        CK(h, cudaFuncSetAttribute(k_force_tile_dense<double, LIST_FWD>, A, smd));
-        CK(h, cudaFuncSetAttribute(k_force_tile<double, LIST_OBS>, A, (int)FORCE_SMEM_MAX));
-        CK(h, cudaFuncSetAttribute(k_force_tile_dense<double, LIST_OBS>, A, (int)FORCE_SMEM_MAX));
-    }
     h->ntiles = (int)torg.size();
     h->frames = FrameTiles{h->frame_org, h->frame_rel, (int)forg.size(), edge, hframe};
     h->tile_shape = S0;
@@ -922,7 +928,7 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
         int dev = 0;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, dev);
         const double e_pp = 2.0 / 3.0 * M_PI * rho_max * P.r_cut * P.r_cut * P.r_cut * 1.15;
-        const size_t smem_big = 200 * 1024;
+        const size_t smem_big = SSA_SMEM_FIT;
         const size_t per = h->mixed ? (sizeof(float4) + sizeof(ff) + 4) : (sizeof(d4) + sizeof(double) + 4);
         for (int t = 0; t < 2; ++t) {
             dpde_handle::SsaCaps& K = h->ssa_caps[t];
@@ -1114,26 +1120,7 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
     CKC(cudaMalloc(&h->lv_off, sizeof(int) * std::max((size_t)h->nbricks * h->ssa_caps[0].stride, (size_t)h->R * h->ssa_caps[1].stride)));
     CKC(cudaMalloc(&h->lv_n, sizeof(int) * (size_t)h->ndom_max));
     CKC(cudaMalloc(&h->ssa_defer, sizeof(int) * (SSA_NLISTS + SSA_NLISTS * (size_t)h->ndom_max)));
-    {
-        size_t ms = 0, mx = 0;
-        for (const auto& K : h->ssa_caps)
-            for (int t = 0; t < 3; ++t) {
-                ms = std::max(ms, ssa_sched_smem(K.scap_s[t], K.ecap_s[t], K.ccap_s[t], K.stride));
-                mx = std::max(mx, h->mixed ? ssa_exec_smem<float>(K.scap_x[t], K.stride) : ssa_exec_smem<double>(K.scap_x[t], K.stride));
-            }
-        const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-        if (h->mixed) {
-            CKC(cudaFuncSetAttribute(k_ssa_sched<float>, A, (int)ms));
-            CKC(cudaFuncSetAttribute(k_ssa_exec<float>, A, (int)mx));
-        } else {
-            CKC(cudaFuncSetAttribute(k_ssa_sched<double>, A, (int)ms));
-            CKC(cudaFuncSetAttribute(k_ssa_exec<double>, A, (int)mx));
-        }
-    }
-    if (h->mixed)
-        CKC(cudaFuncSetAttribute(k_ssa_domains<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, SSA_DOMAIN_SMEM));
-    else
-        CKC(cudaFuncSetAttribute(k_ssa_domains<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, SSA_DOMAIN_SMEM));
+    CKC(h->mixed ? allow_smem<float>() : allow_smem<double>());
     CKC(cudaMalloc(&h->d_bar, sizeof(GridBarrier)));
     CKC(cudaMemset(h->d_bar, 0, sizeof(GridBarrier)));
     for (int m = 0; m < 2; ++m) {
