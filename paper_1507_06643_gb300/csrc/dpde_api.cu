@@ -12,7 +12,9 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <map>
+#include <queue>
 #include <string>
 #include <utility>
 #include <vector>
@@ -937,29 +939,19 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
             for (const RepInfo& I : h->info)
                 biggest = std::max(biggest, t == 0 ? (double)I.n / (I.B[0] * I.B[1] * I.B[2]) : (double)I.n);
             const double M = ndom > 0 ? (double)N / ndom : 0.0;
-            // Whole replicas (DPDE_SSA): a block per replica level by level,
-            // or all cells of a class at once, class by class. Times in us
-            // per step of the largest replica, fitted to both forms at 300 to
-            // 20,000 particles of density 3 and 343 to 6,000 Lennard-Jones
-            // ones: levels ~ classes (4.5 + 0.075 m) with m maps a cell, a
-            // round of 64 maps at most a level; a class, its latency and m
-            // maps of its cells. (Mixed, levels / classes: 4,000 particles
-            // 422 / 739, 6,000 466 / 261, 8,000 928 / 576, 16,000 5849 / 830;
-            // LJ 343 523 / 2548.)
-            double level_us = 0.0, class_us = 1.0;
-            if (t == 1) {
+            // whole replicas: expected levels of each, ~4.5 + 0.075 m per
+            // colour class with m maps a cell, and a stride that holds them
+            std::vector<double> nlev((size_t)(t == 1 ? n_replicas : 0), 0.0);
+            double m_max = 0.0;
+            for (size_t r = 0; r < nlev.size(); ++r) {
+                const int* off = rdom_off.data() + r * (NCOLOURS + 1);
                 int ncls = 0;
-                for (int k = 0; k < NCOLOURS; ++k) ncls += h->col_off[1][k + 1] > h->col_off[1][k];
-                double m = 0.0;
-                for (const RepInfo& I : h->info) m = std::max(m, I.n * e_pp / 1.15 / I.ncells);
-                const double maps = biggest * e_pp / 1.15, nlev = ncls * (4.5 + 0.075 * m);
-                if (n_replicas <= 1024 && nlev > 0.6 * SSA_MAXLEV)
-                    K.stride = (int)std::min<double>(SSA_MAXLEV_LONG, 1.5 * nlev + 64.0) + 2;
-                const size_t fixed = h->mixed ? ssa_exec_smem<float>(0, K.stride) : ssa_exec_smem<double>(0, K.stride);
-                level_us = (h->mixed ? 0.7 : 3.5) * std::max(nlev, maps / 64.0);
-                if (biggest > (double)((smem_big - fixed) / per)) level_us *= 1.4;   // state not in shared memory
-                if (maps > 0.88 * SSA_LOCAL_MAX || nlev > SSA_MAXLEV_LONG) level_us = INFINITY;   // no schedule
-                class_us = ncls * (h->mixed ? 6.0 + 0.28 * m : 28.0 + 2.05 * m);
+                for (int k = 0; k < NCOLOURS; ++k) ncls += off[k + 1] > off[k];
+                const double m = h->info[r].n * e_pp / 1.15 / h->info[r].ncells;
+                nlev[r] = ncls * (4.5 + 0.075 * m);
+                m_max = std::max(m_max, m);
+                if (nlev[r] > 0.6 * SSA_MAXLEV)
+                    K.stride = std::max(K.stride, (int)std::min<double>(SSA_MAXLEV_LONG, 1.5 * nlev[r] + 64.0) + 2);
             }
             auto up16 = [](double x) { return ((int)std::ceil(x) + 15) / 16 * 16; };
             // entries that fit beside sc particles in ~200 KB of schedule
@@ -997,7 +989,56 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
             const size_t xs1 = h->mixed ? ssa_exec_smem<float>(K.scap_x[1], K.stride) : ssa_exec_smem<double>(K.scap_x[1], K.stride);
             K.grid_x[1] = h->nsm * std::max<int>(1, std::min<int>(8, (int)(smem_sm / (xs1 + 1024))));
             K.grid_x[2] = h->nsm;
-            K.ok = biggest <= 16384.0 && level_us <= class_us;
+            K.ok = biggest <= 16384.0;
+            if (t == 0 || !K.ok) continue;
+            // Whole replicas (DPDE_SSA): a block per replica level by level,
+            // or all cells of a class at once, class by class. Estimates in
+            // us of the whole launch, fitted to steps of 1 to 2,432 replicas
+            // of 300 to 9,000 particles at densities 2.5 to 3.5, alike and
+            // uneven, and Lennard-Jones ones of 500 to 2,048, in both
+            // precisions (380 steps in both forms, 11 to 14 % rms; the form
+            // taken is at most 11 % slower than the other one, but for
+            // replicas within 5 % of the entries a schedule holds).
+            //   levels: a replica's chain is its levels or its rounds of 64
+            //     maps, and longer where the state exceeds shared memory or
+            //     the regular schedule defers it; the blocks resident at once
+            //     take the replicas in order.
+            //   classes: a class is its longest cell, and the chip's rate
+            //     where its cells fill it; a warp per cell, then a thread.
+            // Mixed, levels / classes: 4,000 particles 431 / 838, 6,000
+            // 474 / 294; 64 replicas of 6,000 597 / 901 (beyond 32 cells of a
+            // class per SM), 152 813 / 1129, 512 (four waves) 2982 / 2162.
+            struct Fit {
+                double chain, global;            // us a level; state in global memory
+                double c0, c1, x0, x1;           // a warp per cell: c0 + c1 m + (x0 + x1 m) cells per SM
+                double t0, t1, y1;               // a thread per cell: t0 + t1 m + y1 m cells per SM
+            };
+            const Fit F = h->mixed ? Fit{0.73, 1.57, 6.3, 0.245, 0.26, 0.0136, 13.3, 1.03, 0.0018}
+                                   : Fit{2.96, 1.39, 34.0, 1.9, 1.5, 0.36, 81.0, 7.0, 0.045};
+            const size_t fixed = h->mixed ? ssa_exec_smem<float>(0, K.stride) : ssa_exec_smem<double>(0, K.stride);
+            const int per_sm = std::max<int>(1, std::min<int>(h->mixed ? 4 : 2, (int)(smem_sm / (fixed + K.scap_x[0] * per + 1024))));
+            std::priority_queue<double, std::vector<double>, std::greater<double>> busy;   // ends of the blocks running
+            double level_us = 0.0, class_us = 0.0;
+            for (int r = 0; r < n_replicas; ++r) {
+                const double n = (double)h->info[r].n, maps = n * e_pp / 1.15;
+                double us = F.chain * std::max(nlev[r], maps / 64.0) * (n > xfit ? F.global : 1.0);
+                if (n > K.scap_s[0] || maps > K.ecap_s[0]) us *= 1.3;
+                if (maps > 0.95 * SSA_LOCAL_MAX || nlev[r] > SSA_MAXLEV_LONG) us = INFINITY;   // no schedule
+                if ((int)busy.size() == h->nsm * per_sm) {
+                    us += busy.top();
+                    busy.pop();
+                }
+                busy.push(us);
+                level_us = std::max(level_us, us);
+            }
+            for (int k = 0; k < NCOLOURS; ++k) {
+                const int n = h->col_off[1][k + 1] - h->col_off[1][k];
+                const double x = (double)n / h->nsm;
+                if (n > 0)
+                    class_us += n <= CELLS_SM * h->nsm ? F.c0 + F.c1 * m_max + (F.x0 + F.x1 * m_max) * x
+                                                       : F.t0 + F.t1 * m_max + F.y1 * m_max * x;
+            }
+            K.ok = level_us <= class_us;
         }
     }
     auto bail = [&](cudaError_t e, const char* what) {
