@@ -646,6 +646,8 @@ int set_tiles(dpde_handle* h, int edge) {
         S.nhc = (w[0] + 2) * (w[1] + 2) * (w[2] + 2);
         S.noc = w[0] * w[1] * w[2];
         S.wide = mean_frame > 0.5 * hframe;   // some frame tile may go cell by cell
+        const double rc2 = h->prm.r_cut * h->prm.r_cut;
+        S.filter2 = h->mixed || (rc2 >= 0x1p-80 && rc2 <= 0x1p80) ? (float)rc2 * (1.0f + 2e-4f) : NAN;
         return S;
     };
     auto warps = [&](double over) {   // for the mean own particles, times `over`

@@ -238,9 +238,14 @@ constexpr int FORCE_LIST = 32 * FORCE_LSTRIDE;   // entries of a warp's lists
 
 // Shared-memory shape of a launch: halo particles staged (a multiple of 4),
 // halo cells and own cells of the largest work tile; wide: float positions
-// are staged beside the exact ones.
+// are staged beside the exact ones. filter2: square of the filter's radius,
+// which covers the rounding of the float coordinates (under 1e-6 of a tile),
+// far below 1e-4 of the cutoff; NaN, which lets every candidate pass, where
+// the square of a cutoff in FP64 lies near the ends of a float's range (a
+// product by a unit per staged coordinate cost the FP64 pass 4 %).
 struct ForceShape {
     int hcap, nhc, noc, wide;
+    float filter2;
 };
 
 __host__ __device__ inline size_t up_to(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -415,9 +420,7 @@ __device__ __forceinline__ void force_tile_run(const Ctx<T>& C, int tile, const 
         for (int k = b; k < e; ++k) own[at + k - b] = (unsigned short)k;
     }
     __syncthreads();
-    // the filter's radius covers the rounding of the float coordinates
-    // (under 1e-6 of a tile), far below 1e-4 of the cutoff
-    const float wide2 = (float)C.rc2 * (1.0f + 2e-4f);
+    const float wide2 = S.filter2;
     const T near2 = C.rc2 * (T)(1.0 - 1e-5);
     const bool fast = !fr.rel && C.pot.kind == 0;
     // 5. a thread per own particle
@@ -435,7 +438,7 @@ __device__ __forceinline__ void force_tile_run(const Ctx<T>& C, int tile, const 
         auto near = [&](int j) {
             const float4 c = fq[j];
             const float dx = fi.x - c.x, dy = fi.y - c.y, dz = fi.z - c.z;
-            return dx * dx + dy * dy + dz * dz < wide2;
+            return !(dx * dx + dy * dy + dz * dz >= wide2);
         };
         PairOut<T> o = pair_out(C, i);
         // the listed candidates of my particle, n of them, in the exact
