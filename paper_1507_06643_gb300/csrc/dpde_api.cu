@@ -618,15 +618,27 @@ int set_tiles(dpde_handle* h, int edge) {
                                           (double)((200 * 1024 - thead) / tper)) & ~3;
     const int hframe = std::max(fit, (int)std::min<double>(std::min<double>(2.5 * mean_frame + 64.0, 65535.0),
                                                     (double)((224 * 1024 - thead) / tper))) & ~3;
-    // work tile: edge x edge x 2 cells in a single box (the least halo per
-    // own particle: force pass 720 us at 4M against 800 us with 3 x 3 x 3),
-    // 3 x 3 x 3 in a batch, whose smaller boxes the frames cut into narrow
-    // remainders (256 boxes of 2,000 to 64,000: 1085 us against 1240 us). Its
-    // longest edge is halved while the mean halo takes more than ~1/4 of an
-    // SM's shared memory or the launch has fewer than six blocks per SM
-    // (108,000 particles: 43 -> 38 us with the first halving).
-    int w[3] = {edge, edge, std::min(2, edge)};
-    if (h->R > 1) w[0] = w[1] = w[2] = (edge + 1) / 2;
+    // work tile: the whole frame tile where its mean own particles are few
+    // (at most 144: what is read per cell of the halo then bounds the pass),
+    // else a slab of it, down to edge x edge x 2 cells, in a single box (the
+    // least halo per own particle: force pass 720 us at 4M against 800 us with
+    // 3 x 3 x 3) and 3 x 3 x 3 in a batch of boxes beyond 4 cells, which the
+    // frames cut into narrow remainders (256 boxes of 2,000 to 64,000: 1085 us
+    // against 1240 us). Its longest edge is halved while the mean halo takes more than
+    // ~1/4 of an SM's shared memory or the launch has fewer than six blocks
+    // per SM (108,000 particles: 43 -> 38 us with the first halving).
+    // Sparse systems, whole frames against the slabs of 2 and the 3 x 3 x 3:
+    // 300,000 particles at density 0.02 497 us against 802, at 0.5 52 against
+    // 70 (at 1.5 58 against 55), 200 boxes of 3,000 at 0.3 133 against 319;
+    // boxes of 4 x 4 x 4 cells (300 of 200 particles) 25 against 39.
+    int ext[3] = {1, 1, 1};   // the largest frame tile
+    for (const RepInfo& I : h->info)
+        for (int a = 0; a < 3; ++a) ext[a] = std::max(ext[a], std::min(edge, I.nc[a]));
+    int w[3] = {ext[0], ext[1], ext[2]};
+    auto own = [&]() { return h->per_cell_max * w[0] * w[1] * w[2]; };
+    for (int p = 2; own() > 144.0 && w[2] > 2; ++p) w[2] = ceil_div(ext[2], p);
+    if (h->R > 1 && own() > 144.0 && std::max(ext[0], std::max(ext[1], ext[2])) > 4)
+        for (int a = 0; a < 3; ++a) w[a] = std::min(ext[a], (edge + 1) / 2);
     auto count = [&]() {
         long long n = 0;
         for (const RepInfo& I : h->info) {
@@ -651,8 +663,7 @@ int set_tiles(dpde_handle* h, int edge) {
         return S;
     };
     auto warps = [&](double over) {   // for the mean own particles, times `over`
-        const double own = h->per_cell_max * w[0] * w[1] * w[2] * over;
-        return std::max(2, std::min(FORCE_WARPS_MAX, (int)std::ceil(own / 32.0)));
+        return std::max(2, std::min(FORCE_WARPS_MAX, (int)std::ceil(own() * over / 32.0)));
     };
     auto bytes = [&](const ForceShape& S, double over = 1.08) {
         return h->mixed ? force_smem<float>(S, warps(over)) : force_smem<double>(S, warps(over));
@@ -661,7 +672,7 @@ int set_tiles(dpde_handle* h, int edge) {
     const size_t budget = h->mixed ? 56 * 1024 : 74 * 1024;
     for (;;) {
         const bool big = bytes(shape(1.08 * mean_halo() + 64.0)) > budget;
-        const bool few = count() < 6 * nsm && h->per_cell_max * w[0] * w[1] * w[2] > 24.0;
+        const bool few = count() < 6 * nsm && own() > 24.0;
         const int a = w[1] >= w[0] && w[1] >= w[2] ? 1 : (w[0] >= w[2] ? 0 : 2);
         if (!(big || few) || w[a] == 1) break;
         w[a] = (w[a] + 1) / 2;
