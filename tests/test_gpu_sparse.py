@@ -4,9 +4,10 @@ a sparse box in one handle. Two SER steps against the oracle, element by
 element, with the tolerances of the parity tests (1e-11 in FP64, 2e-5 mixed:
 double and float rounding of the pair arithmetic, accumulated over two
 steps)."""
+import numpy as np
 import pytest
 
-from gpu_util import assert_parity
+from gpu_util import assert_parity, run_both
 
 pytestmark = pytest.mark.gpu
 
@@ -24,3 +25,33 @@ def test_sparse_boxes(boxes, precision):
     specs = [(n, box, 50.0, 1.0, (1, 1, 1)) for n, box in boxes]
     for _ in assert_parity(specs, precision, "SER", 2, TOL[precision], (3,), dt=0.002):
         pass
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("bricks,walls", [((1, 1, 1), (0, 0.0)), ((7, 5, 4), (0, 0.0)), ((1, 1, 1), (1, -0.5))])
+def test_observables_of_a_very_sparse_box(bricks, walls, precision):
+    """950,000 cells for 3,000 particles, half of them in a drop across the
+    periodic corner: the pair sums particle by particle, rows of cells that
+    are neighbours in memory and rows that a domain or the box cuts, against
+    the oracle (the parity tolerance, on sums: relative to the sum)."""
+    box = (101.0, 97.5, 99.2)
+    rng = np.random.default_rng(11)
+    n = 3000
+    q = rng.random((n, 3)) * np.asarray(box)
+    q[:n // 2] = (rng.random((n // 2, 3)) - 0.5) * 8.0
+    if walls[0]:
+        q[:n // 2, 2] += 4.0
+    q = np.mod(q, np.asarray(box))
+    p = rng.standard_normal((n, 3))
+    if precision == "mixed":
+        q = q.astype(np.float32).astype(np.float64)
+        p = p.astype(np.float32).astype(np.float64)
+        q = np.where(q >= np.asarray(box), 0.0, q)
+    e = 50.0 * (1 + 0.05 * rng.uniform(-1, 1, n))
+    errs, _, (_, _, _, obs), ref = run_both([(n, box, 50.0, 1.0, bricks)], precision, "SER", 1, dt=0.002,
+                                            state=(q, p, e), walls=walls)
+    assert max(errs.values()) < TOL[precision], errs
+    o = ref.observables(0)
+    assert o["U"] > 100.0
+    for k in ("U", "Tpot_num", "Tpot_den"):
+        assert abs(obs[0][k] - o[k]) <= 10 * TOL[precision] * abs(o[k]), (k, obs[0][k], o[k])
