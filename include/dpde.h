@@ -394,8 +394,9 @@ typedef struct dpde_tuning {
                          /* memory (maps of one level share no particle); used where  */
                          /* no domain is expected above 16,384 particles and, for     */
                          /* DPDE_SSA, where it is expected to be the faster, else 0.  */
-                         /* 0: one launch per colour class, a warp per cell, or a      */
-                         /* thread per cell of a class of more than 32 cells per SM;  */
+                         /* 0: one launch per colour class, a warp per cell, or a     */
+                         /* thread per cell of a class of more than 32 cells per SM   */
+                         /* and in sparse systems;                                    */
                          /* 1 (Hybrid only, DPDE_SSA then takes 0): one launch in     */
                          /* which each warp takes whole domains and walks their       */
                          /* colour classes in order (domains share no chain, so their */

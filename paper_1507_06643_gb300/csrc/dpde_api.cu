@@ -58,7 +58,12 @@ constexpr size_t SSA_ALONE_SMEM = 116 * 1024;   // one such block per SM
 // that of the longest cell, ~10 us, until the warps fill the chip (SSA step at
 // density 3: 20,011 particles 442 -> 280 us, 64,000 642 -> 406, 200,000, 16
 // cells per SM, 898 -> 655; 1,000,000, 81 per SM, 1177 against 1764).
+// A cell of few maps is done sooner by its thread than a warp has staged it:
+// from this many maps a cell, mixed and FP64 (mixed, phase of 40,000 particles
+// by threads / warps, 0.5 maps a cell 303 / 404 us, 1.1 363 / 403, 2.1 296 /
+// 290, 5.2 809 / 684; FP64 0.2 434 / 452, 0.5 871 / 851, 2.1 1190 / 967).
 constexpr int CELLS_SM = 32;
+constexpr double CELLS_MAPS_MIXED = 1.6, CELLS_MAPS_FP64 = 0.4;
 constexpr int STATE_CHUNKS = 4;   // chunks of a host <-> device state transfer
 
 struct dpde_handle {
@@ -126,6 +131,7 @@ struct dpde_handle {
     GridBarrier* d_bar = nullptr;
     long long wait_budget = 2000000000ll;
     int cells_lcap = 16;      // particles staged by a warp of k_ssa_cells
+    int cells_max = 0;        // cells of a class up to which a warp takes a cell
     int ssa_group = 0;        // bricks per warp; 0 = dom_group_auto
     int dom_group_auto = 1;   // 32 / the largest class of a brick, in 1..SSA_GROUP_MAX
     ForceShape tile_shape{}, tile_shape_dense{};   // shared-memory shapes of the two force launches
@@ -396,7 +402,7 @@ void enqueue_ssa(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T dt, T sqrt_
     for (int k = 0; k < NCOLOURS; ++k) {
         const int n = off[k + 1] - off[k];
         if (n == 0) continue;
-        if (n <= CELLS_SM * h->nsm)
+        if (n <= h->cells_max)
             k_ssa_cells<T><<<n, 32, ssa_cells_smem<T>(h->cells_lcap), st>>>(C, h->col_cells[whole] + off[k], whole,
                                                                           h->cells_lcap, dt, sqrt_dt);
         else
@@ -948,6 +954,8 @@ int dpde_create(const dpde_params* params, int32_t n_replicas, const dpde_replic
         int dev = 0;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, dev);
         const double e_pp = 2.0 / 3.0 * M_PI * rho_max * P.r_cut * P.r_cut * P.r_cut * 1.15;
+        const double maps_cell = e_pp / 1.15 * per_cell_max;
+        h->cells_max = maps_cell >= (h->mixed ? CELLS_MAPS_MIXED : CELLS_MAPS_FP64) ? CELLS_SM * h->nsm : 0;
         const size_t smem_big = SSA_SMEM_FIT;
         const size_t per = h->mixed ? (sizeof(float4) + sizeof(ff) + 4) : (sizeof(d4) + sizeof(double) + 4);
         for (int t = 0; t < 2; ++t) {

@@ -1,7 +1,7 @@
 """The forms of the SSA against one another where each can go wrong (GPU), with
 the launch counts that tell which form ran: cells of more than 32 particles in
 a warp's rows, a domain of hundreds of chunks whose state exceeds shared
-memory, classes of more than 32 cells per SM (a thread per cell).
+memory, classes of more than 32 cells per SM (a thread per cell), sparse
 systems (cells too empty for a warp). The reference is the persistent launch
 (ssa_mode 3: each cell's chain by one thread, a grid barrier between classes).
 Two steps, bit for bit."""
@@ -20,6 +20,8 @@ CASES = {
     # 110,592 cells in 18 classes of 6,144, on at most 152 SMs
     "large_classes": (331776, (48.1, 48.1, 48.1), (8, 8, 8), "HYBRID", 0.01, True),
     "large_replica": (400000, (52.3, 51.2, 50.4), (1, 1, 1), "SSA", 0.01, False),
+    "sparse": (3000, (24.7, 25.2, 23.9), (1, 1, 1), "SSA", 0.01, True),
+    "sparse_domains": (3000, (24.7, 25.2, 23.9), (2, 3, 2), "HYBRID", 0.01, True),
 }
 
 
