@@ -690,13 +690,17 @@ int set_tiles(dpde_handle* h, int edge) {
     }
     const size_t smem_limit = FORCE_SMEM_MAX;
     // regular capacity 1.08x the mean halo + 64 (over 4 standard deviations
-    // of a uniform fluid's count), deferred tiles 2.5x the mean
+    // of a uniform fluid's count), deferred tiles 2.5x the mean, or what four
+    // blocks per SM hold: beyond, a tile goes through global memory (40,500
+    // particles, 15 % of them at 3.2 times the mean, SER step 538 -> 117 us)
     auto capped = [&](double halo) {
         ForceShape S = shape(halo);
         while (S.hcap > 64 && bytes(S, 1.7) > smem_limit) S.hcap = (S.hcap * 15 / 16) & ~3;
         return S;
     };
-    const ForceShape S0 = capped(1.08 * mean_halo() + 64.0), S1 = capped(2.5 * mean_halo() + 128.0);
+    const ForceShape S0 = capped(1.08 * mean_halo() + 64.0);
+    ForceShape S1 = capped(2.5 * mean_halo() + 128.0);
+    while (bytes(S1, 1.7) + 64 * 56 <= 55 * 1024) S1.hcap += 64;   // (at most 56 bytes a particle)
     const size_t smem_dense = bytes(S1, 1.7);
     std::vector<int4> torg, tdim, forg;
     for (int r = 0; r < h->R; ++r) {

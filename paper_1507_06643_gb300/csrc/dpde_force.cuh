@@ -353,10 +353,12 @@ __device__ __forceinline__ void force_tile_run(const Ctx<T>& C, int tile, const 
             if (tid == 0) defer[atomicAdd(ndefer, 1)] = tile;
             return;
         }
-        for (int c = tid; c < nown; c += blockDim.x) {
+        // eight threads an own cell (one left most of the block idle)
+        for (int u = tid; u < nown << 3; u += blockDim.x) {
+            const int c = u >> 3;
             const int h = ((c / (dim.x * dim.y) + 1) * HY + (c / dim.x) % dim.y + 1) * HX + c % dim.x + 1;
             const int g = cinfo[h].x, n = hstart[h + 1] - hstart[h];
-            for (int k = 0; k < n; ++k) force_one_global<T, LM>(C, g + k, fr, half_dt, kick);
+            for (int k = u & 7; k < n; k += 8) force_one_global<T, LM>(C, g + k, fr, half_dt, kick);
         }
         return;
     }
