@@ -630,8 +630,8 @@ int set_tiles(dpde_handle* h, int edge) {
     const int hframe = std::max(fit, (int)std::min<double>(std::min<double>(2.5 * mean_frame + 64.0, 65535.0),
                                                     (double)((224 * 1024 - thead) / tper))) & ~3;
     // work tile: the whole frame tile where its mean own particles are few
-    // (at most 144: what is read per cell of the halo then bounds the pass),
-    // else a slab of it, down to edge x edge x 2 cells, in a single box (the
+    // (at most 144: what is read per cell of the halo then bounds the pass)
+    // and six blocks per SM are left, else a slab of it, down to edge x edge x 2 cells, in a single box (the
     // least halo per own particle: force pass 720 us at 4M against 800 us with
     // 3 x 3 x 3) and 3 x 3 x 3 in a batch of boxes beyond 4 cells, which the
     // frames cut into narrow remainders (256 boxes of 2,000 to 64,000: 1085 us
@@ -647,9 +647,6 @@ int set_tiles(dpde_handle* h, int edge) {
         for (int a = 0; a < 3; ++a) ext[a] = std::max(ext[a], std::min(edge, I.nc[a]));
     int w[3] = {ext[0], ext[1], ext[2]};
     auto own = [&]() { return h->per_cell_max * w[0] * w[1] * w[2]; };
-    for (int p = 2; own() > 144.0 && w[2] > 2; ++p) w[2] = ceil_div(ext[2], p);
-    if (h->R > 1 && own() > 144.0 && std::max(ext[0], std::max(ext[1], ext[2])) > 4)
-        for (int a = 0; a < 3; ++a) w[a] = std::min(ext[a], (edge + 1) / 2);
     auto count = [&]() {
         long long n = 0;
         for (const RepInfo& I : h->info) {
@@ -663,6 +660,9 @@ int set_tiles(dpde_handle* h, int edge) {
         }
         return n;
     };
+    for (int p = 2; (own() > 144.0 || count() < 6 * nsm) && w[2] > 2; ++p) w[2] = ceil_div(ext[2], p);
+    if (h->R > 1 && own() > 144.0 && std::max(ext[0], std::max(ext[1], ext[2])) > 4)
+        for (int a = 0; a < 3; ++a) w[a] = std::min(ext[a], (edge + 1) / 2);
     auto shape = [&](double halo) {
         ForceShape S;
         S.hcap = (int)std::min(halo, 65000.0) & ~3;
