@@ -381,9 +381,36 @@ def run_ours(args):
             out["parity"] = parity_report(w, base, args.scheme)
             if args.batched_steps > 0:
                 out["cpu_baseline_batched"] = cpu_batched_baseline()
-        print(json.dumps(out))
+        if args.report:
+            with open(args.report, "w") as f:
+                json.dump(out, f)
+        print(json.dumps(line_of(out)))
     if world > 1:
         tdist.destroy_process_group()
+
+
+def six_digits(x):
+    """x with its floats cut to six significant digits."""
+    if isinstance(x, dict):
+        return {k: six_digits(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [six_digits(v) for v in x]
+    return float(f"{x:.6g}") if isinstance(x, float) and math.isfinite(x) else x
+
+
+def line_of(out):
+    """What the JSON line says of the result `out`: without the shock's profile,
+    the descriptions of the legs' samples and what the phases' rooflines share
+    with the step's, nested floats at six digits. A reader of a job's output
+    may keep only its last few kilobytes; with the profile the line had 27."""
+    line = {}
+    for key, v in out.items():
+        if key == "roofline_phases":
+            v = {ph: {"kernel": r["kernel"], "frac": r["frac"]} for ph, r in v.items()}
+        elif isinstance(v, dict) and key != "config":
+            v = {k: x for k, x in v.items() if k not in ("eps_profile", "sample", "note", "tuning")}
+        line[key] = six_digits(v) if isinstance(v, dict) else v
+    return line
 
 
 def fp64_run(args, spec_reps, w, q, p, e, stream):
@@ -473,12 +500,28 @@ def drift_run(args, stream):
     return out
 
 
+SHOCK_SLABS = 800   # of the shock's profile
+
+
+def slab_means(z, e, length, slabs):
+    """Mean of e over the particles of each of `slabs` equal slabs of [0, length) (0 where there are none)."""
+    idx = np.minimum((z / length * slabs).astype(np.int64), slabs - 1)
+    cnt = np.bincount(idx, minlength=slabs)
+    return np.bincount(idx, weights=e, minlength=slabs) / np.maximum(cnt, 1)
+
+
+def eps_profile(states, length, times, slabs):
+    """The profiles of (name, z, eps) states."""
+    return {"slabs": slabs, "slab_width": length / slabs, "times": times,
+            **{k: [round(float(x), 3) for x in slab_means(z, e, length, slabs)] for k, z, e in states}}
+
+
 def shock_run(args, stream):
     """The shock workload (BASELINE config 4: box 40 x 40 x 800 at density 3,
     halves at +-2 along z, C_v = 100, dt = 0.005, mixed precision, Hybrid):
     throughput, total-energy drift over --shock-steps steps, and the mean
-    internal energy in 800 slabs along z at the start, halfway and at the
-    end (the analogue of the eps profiles of Sec. V)."""
+    internal energy in slabs along z at the start, halfway and at the end
+    (the analogue of the eps profiles of Sec. V)."""
     import torch
     from paper_1507_06643_gb300 import dpde, inputs
     w = inputs.shock_40x40x800("mixed")
@@ -489,17 +532,14 @@ def shock_run(args, stream):
     S.set_state(q, p, e)
     S.step(3, w.dt, "HYBRID")
     S.sync()
-    nsl = 800
     Lz = spec.box[2]
 
-    def profile():
+    def state(name):
         qq, _, ee = S.get_state()
-        idx = np.minimum((qq[:, 2] / Lz * nsl).astype(np.int64), nsl - 1)
-        cnt = np.bincount(idx, minlength=nsl)
-        return np.bincount(idx, weights=ee, minlength=nsl) / np.maximum(cnt, 1)
+        return name, qq[:, 2], ee
 
     o0 = S.observables(check=False)[0]
-    prof = {"t0": profile()}
+    states = [state("t0")]
     half = args.shock_steps // 2
     t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     torch.cuda.synchronize()
@@ -508,18 +548,17 @@ def shock_run(args, stream):
     t1.record(stream)
     t1.synchronize()
     ms = t0.elapsed_time(t1)
-    prof["half"] = profile()
+    states.append(state("half"))
     S.step(args.shock_steps - half, w.dt, "HYBRID")
     status = S.sync()
     o1 = S.observables(check=False)[0]
-    prof["end"] = profile()
+    states.append(state("end"))
     S.close()
+    times = [0.0, half * w.dt, args.shock_steps * w.dt]
     return {"workload": w.name, "n": spec.n, "dt": w.dt, "steps": args.shock_steps, "scheme": "HYBRID",
             "precision": "mixed", "value": spec.n * half / (ms / 1e3), "unit": UNIT, "timed_steps": half,
             "ms_per_step": ms / half, "rel_drift": abs(o1["E"] - o0["E"]) / abs(o0["E"]), "status": status,
-            "neg_eps": o1["neg_eps"], "eps_profile": {"slabs": nsl, "slab_width": Lz / nsl,
-                                                      "times": [0.0, half * w.dt, args.shock_steps * w.dt],
-                                                      **{k: [round(float(x), 3) for x in v] for k, v in prof.items()}}}
+            "neg_eps": o1["neg_eps"], "eps_profile": eps_profile(states, Lz, times, SHOCK_SLABS)}
 
 
 def batched_run(args, stream):
@@ -791,6 +830,8 @@ def main():
     ap.add_argument("--scheme", default="HYBRID", choices=["SER", "HYBRID", "SEM", "SSA"])
     ap.add_argument("--precision", default="mixed", choices=["mixed", "fp64"])
     ap.add_argument("--profile-steps", type=int, default=10)
+    ap.add_argument("--report", metavar="FILE", help="write everything measured to FILE: the JSON line with all "
+                    "digits, the rooflines' peaks and the shock's internal-energy profile")
     ap.add_argument("--e2e-steps", type=int, default=10)
     ap.add_argument("--cpu-seconds", type=float, default=15.0)
     ap.add_argument("--no-cpu-baseline", action="store_true")
