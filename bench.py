@@ -142,7 +142,7 @@ OPS_PER_PAIR = {"ssa": 95.0, "ssa_gauss": OPS_GAUSS, "sweep1": OPS_GAUSS + 40.0,
 # execution kernel; its "ssa_gauss" phase is the level schedule, which has no
 # algorithmic operations of its own (it orders the pairs)
 OPS_PER_PAIR_LEVELS = {"ssa": 95.0 + OPS_GAUSS}
-KERNEL_OF_PHASE = {"ssa": "k_ssa_colour", "ssa_gauss": "k_ssa_gauss", "sweep1": "k_ser_sweep1",
+KERNEL_OF_PHASE = {"ssa": "k_ssa_cells / k_ssa_colour", "ssa_gauss": "k_ssa_gauss", "sweep1": "k_ser_sweep1",
                    "sweep2": "k_ser_sweep2", "force": "k_force_tile", "gather": "k_rank_gather",
                    "kick_drift": "k_kick_drift_key"}
 
@@ -216,6 +216,21 @@ def step_roofline(w, scheme, ms_step, peaks, peak_src):
             "measured_us": ms_step * 1e3, "frac": model_s / (ms_step / 1e3),
             "ops_per_particle": ops / n, "bytes_per_particle": nbytes / n,
             "peak_source": f"{peak_src} hbm_gbs; 152 SMs x 128 lanes x {clk_mhz:.0f} MHz"}
+
+
+def ssa_form(S, scheme, mode):
+    """The form of the SSA launches that runs under the tuning's ssa_mode: DPDE_SSA
+    has no per-domain launch (1), and 2 takes the class launches (0) where the
+    library expects those to be the faster ones or a domain is too large."""
+    if mode == 1 and scheme == "SSA":
+        return 0
+    if mode != 2 or scheme not in ("HYBRID", "SSA"):
+        return mode
+    levels = S.step_launches(scheme)
+    S.set_tuning(ssa_mode=0)
+    classes = S.step_launches(scheme)
+    S.set_tuning(ssa_mode=2)
+    return 0 if levels == classes else 2
 
 
 def run_ours(args):
@@ -299,7 +314,7 @@ def run_ours(args):
            "d2h_bytes_per_step": int(q.nbytes + p.nbytes + e.nbytes), "status": e2e_status}
 
     peaks, peak_src = measured_peaks()
-    mode = tuning.get("ssa_mode")
+    mode = ssa_form(S, args.scheme, tuning["ssa_mode"])
 
     def phase_roofline(ph, secs=None):
         bound, work, unit = algorithmic_model(w, ph, args.scheme, w.precision, mode)

@@ -1,6 +1,6 @@
 """What the benchmark prints of its result: a line short enough for a reader
-that keeps a few kilobytes of it, with every key, and the shock's profile, which
-only the report holds. CPU only."""
+that keeps a few kilobytes of it, with every key, the shock's profile, which
+only the report holds, and the form of the SSA that ran. CPU only."""
 import json
 import sys
 from pathlib import Path
@@ -43,3 +43,25 @@ def test_line_is_short_and_keeps_its_keys():
     assert line["value"] == out["value"] and line["config"] == out["config"]
     assert line["shock"] == {"value": 333333000.0} and line["parity"] == {"fp64": 3.33333e-14}
     assert line["roofline_phases"]["0"] == {"kernel": "k", "frac": 0.333333}
+
+
+class Launches:
+    """A handle whose level form is possible or not."""
+
+    def __init__(self, levels):
+        self.levels, self.mode = levels, 2
+
+    def set_tuning(self, ssa_mode):
+        self.mode = ssa_mode
+
+    def step_launches(self, scheme):
+        return 16 if self.mode == 2 and self.levels else 35
+
+
+def test_the_form_that_runs():
+    for levels, form in ((True, 2), (False, 0)):
+        S = Launches(levels)
+        assert bench.ssa_form(S, "SSA", 2) == form and S.mode == 2
+    assert bench.ssa_form(Launches(True), "SSA", 1) == 0
+    assert bench.ssa_form(Launches(True), "HYBRID", 1) == 1
+    assert bench.ssa_form(Launches(False), "SER", 2) == 2
