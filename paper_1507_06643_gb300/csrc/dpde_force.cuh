@@ -423,7 +423,6 @@ __device__ __forceinline__ void force_tile_run(const Ctx<T>& C, int tile, const 
     }
     __syncthreads();
     const float wide2 = S.filter2;
-    const T near2 = C.rc2 * (T)(1.0 - 1e-5);
     const bool fast = !fr.rel && C.pot.kind == 0;
     // 5. a thread per own particle
     const int no = s_row[nrow];
@@ -460,7 +459,6 @@ __device__ __forceinline__ void force_tile_run(const Ctx<T>& C, int tile, const 
                     }
                     const int cj = cinfo[cell[hj]].y;
                     const int dx = (cj & 15) - icx, dy = ((cj >> 4) & 15) - icy, dz = (cj >> 8) - icz;
-                    hit = hit && abs(dx) <= 1 && abs(dy) <= 1 && abs(dz) <= 1;
                     ddx -= shift<T>(dx, lx);
                     ddy -= shift<T>(dy, ly);
                     ddz -= shift<T>(dz, lz);
@@ -469,16 +467,7 @@ __device__ __forceinline__ void force_tile_run(const Ctx<T>& C, int tile, const 
                 hit = hit && r2 < C.rc2;
                 T ir = rsqrt_normal(r2);
                 bool sum = true;
-                if (hit && !(r2 >= min_normal<T>() && r2 <= near2)) {   // rare
-                    if (r2 > near2) {
-                        // a particle two cells off can only round into reach
-                        // where a cell is hardly wider than the cutoff
-                        const int cj = cinfo[cell[hj]].y;
-                        hit = abs((cj & 15) - icx) <= 1 && abs(((cj >> 4) & 15) - icy) <= 1 && abs((cj >> 8) - icz) <= 1;
-                    } else {
-                        sum = close_pair(C, r2, ir, o);
-                    }
-                }
+                if (hit && !(r2 >= min_normal<T>())) sum = close_pair(C, r2, ir, o);   // rare
                 const int j = slot_bits(qj);
                 force_hit<T, LM, PLAIN>(C, hit, sum, j, hj > hi, (unsigned)(j - br.x) >= (unsigned)br.y, ddx, ddy, ddz,
                                         r2, ir, o);
