@@ -248,8 +248,6 @@ struct ForceShape {
     float filter2;
 };
 
-__host__ __device__ inline size_t up_to(size_t x, size_t a) { return (x + a - 1) / a * a; }
-
 template <class T>
 __host__ __device__ inline size_t force_smem(const ForceShape& S, int warps) {
     return (size_t)S.hcap * (sizeof(vec_t<T>) + (sizeof(T) != 4 || S.wide ? 16 : 0) + 2 + 2) + (size_t)(S.nhc + S.noc) * 8 +

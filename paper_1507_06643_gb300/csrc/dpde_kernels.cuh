@@ -1349,13 +1349,6 @@ __global__ void __launch_bounds__(SSA_THREADS_MAX) k_ssa_domains(Ctx<T> C, const
     }
 }
 
-template <class T>
-__global__ void k_refresh_beta(Ctx<T> C) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= C.N) return;
-    C.pB[s].w = beta_of(C.eB[s], C.reps[C.rep_of_slot[s]]);
-}
-
 __global__ void k_step_inc(long long* step) { *step += 1; }
 
 // ---------------------------------------------------------------------------
