@@ -147,10 +147,9 @@ KERNEL_OF_PHASE = {"ssa": "k_ssa_cells / k_ssa_colour", "ssa_gauss": "k_ssa_gaus
                    "kick_drift": "k_kick_drift_key"}
 
 # DRAM bytes (read + write) per launch of a kernel from an ncu capture of the
-# named configuration with the caches kept warm
-# (profiles/launches_large_n4m_hybrid_mixed.md); reported only for that
-# configuration and kernel.
-MEASURED_TRAFFIC = {("large_n4m", "HYBRID", "mixed", "k_ssa_colour", 5): 168.6e6}
+# named configuration and tile edge with the caches kept warm
+# (profiles/k_force_tile_medium_n1m.md); reported only for those.
+MEASURED_TRAFFIC = {("large_n4m", "HYBRID", "mixed", "k_force_tile", 6): 1.031e9}
 
 
 def pair_counts(w):

@@ -379,8 +379,9 @@ int dpde_set_projection(dpde_handle* h, int32_t enable, const double* E0);
  * nothing in the results. */
 typedef struct dpde_tuning {
     int32_t tile_edge;   /* force tile edge in cells, 2..8 (default 6)                */
-    int32_t block;       /* threads per block of the per-particle kernels: a multiple  */
-                         /* of 32 in 64..1024 (default 256)                           */
+    int32_t block;       /* threads per block of the sort, copy and state kernels (the */
+                         /* sweeps' are of 128): a multiple of 32 in 64..1024         */
+                         /* (default 256)                                             */
     int32_t ssa_block;   /* threads per block of the per-class SSA launches, and       */
                          /* threads of a block of the level form's execution that     */
                          /* apply maps (64 more draw the Gaussians): 32, 64, 96 or    */

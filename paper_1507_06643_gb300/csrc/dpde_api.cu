@@ -293,9 +293,10 @@ void enqueue_ssa_levels(dpde_handle* h, const Ctx<T>& C, cudaStream_t st, T dt, 
     V.lv_n = h->lv_n;
     V.stride = K.stride;
     V.rec = reinterpret_cast<SsaRec<T>*>(h->fwd_g);   // (unused by this form: the forward entries' Gaussians)
-    // counts: [0, 1] schedule tiers 1, 2; [2, 3] execution tiers 1, 2 of the
-    // domains the regular schedule kept; [4, 5] execution tiers 1, 2 of those
-    // it deferred; then the lists (the sort has cleared the counts)
+    // counts: [0, 1] what the regular schedule and its tier 1 deferred; [2, 3]
+    // what the regular execution and its tier 1 deferred; [4] what tier 1 of
+    // the execution of list 0 deferred; then the lists (the sort has cleared
+    // the counts)
     int* cnt = h->ssa_defer;
     int* lst[SSA_NLISTS];
     for (int k = 0; k < SSA_NLISTS; ++k) lst[k] = cnt + SSA_NLISTS + (size_t)k * h->ndom_max;

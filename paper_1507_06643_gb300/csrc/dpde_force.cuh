@@ -217,13 +217,13 @@ __device__ void force_one_global(const Ctx<T>& C, int i, const ForceFrame& fr, T
 // listed (12.6 of ~94 at density 3, and the particle itself); the listed ones
 // are then tested and computed in the exact arithmetic, in list order, so
 // sums and lists come out in the order of a plain walk, the warp going
-// through its lists together and without branches (~40 warp instructions a
-// particle, the candidate tests ~115 on 19 of 32 lanes -- the rows of
-// neighbouring cells differ in length -- and the staging ~28).
+// through its lists together and without branches. At 1M and density 3: 161
+// warp instructions a particle on 25 of 32 lanes (the rows of neighbouring
+// cells differ in length), 72 % of the issue slots at four blocks an SM.
 //
 // Measured against one block per frame tile with hits processed row by row:
-// 4M at density 3 (Hybrid) 834 -> 720 us, SER lists at 1M 207 -> 180 us,
-// 108,000 particles 61 -> 39 us, 1,000 in FP64 484 -> 44 us (one tile took
+// 4M at density 3 (Hybrid) 834 -> 644 us, SER lists at 1M 207 -> 176 us,
+// 108,000 particles 61 -> 38 us, 1,000 in FP64 484 -> 44 us (one tile took
 // them all, on one SM); Lennard-Jones at 18 particles a cell, whose frame
 // tiles fit no SM and went particle by particle through global memory,
 // 30.5 ms -> 0.22 ms.
